@@ -23,9 +23,9 @@ struct gs_opt {
     int device = -1;
     int64_t n_rows = 0;
     int64_t capacity = 0;         // rows the current state buffers hold
-    void *m = nullptr, *v = nullptr;
+    void *m = nullptr;            // state rows (m and v of a primitive side by side)
     int64_t capacity2 = 0;        // rows the spare (re-index target) buffers hold
-    void *m2 = nullptr, *v2 = nullptr;
+    void *m2 = nullptr;
     double *tab1 = nullptr, *tab2 = nullptr;
     float2 *fac = nullptr;
     int32_t tab_len = 0;
@@ -62,13 +62,15 @@ size_t state_row_bytes(int prec)
                                    : gs::kRowBytesHyb;
 }
 
-// Bytes of one moment's state for `rows` rows: the rows, and for FP8 the
-// block scales after them (64 floats per 256 rows, from a 256-B boundary).
-size_t fp8_scale_offset(int64_t rows) { return ((size_t)rows * gs::kRowBytesF8 + 255) / 256 * 256; }
+// Bytes of the state of `rows` rows: an m and a v row each, and for FP8 the
+// block scales of m, then of v, after them (64 floats each per 256 rows, from
+// a 256-B boundary).
+size_t fp8_scale_offset(int64_t rows) { return ((size_t)rows * 2 * gs::kRowBytesF8 + 255) / 256 * 256; }
+size_t fp8_scale_floats(int64_t rows) { return (size_t)((rows + gs::kF8BlockRows - 1) / gs::kF8BlockRows) * 64; }
 size_t state_bytes(int prec, int64_t rows)
 {
-    if (prec != GS_MOM_FP8E4M3) return state_row_bytes(prec) * (size_t)rows;
-    return fp8_scale_offset(rows) + (size_t)((rows + gs::kF8BlockRows - 1) / gs::kF8BlockRows) * 64 * sizeof(float);
+    if (prec != GS_MOM_FP8E4M3) return 2 * state_row_bytes(prec) * (size_t)rows;
+    return fp8_scale_offset(rows) + 2 * fp8_scale_floats(rows) * sizeof(float);
 }
 float *fp8_scales(void *base, int64_t capacity)
 {
@@ -192,32 +194,29 @@ int32_t table_length(double b1, double b2)
     return kMaxTable;
 }
 
-// Allocate the m, v rows of `rows` primitives; on failure nothing stays
+// Allocate the state rows of `rows` primitives; on failure nothing stays
 // allocated.
-gs_status alloc_state(gs_opt *o, int64_t rows, void **m, void **v)
+gs_status alloc_state(gs_opt *o, int64_t rows, void **m)
 {
-    const size_t bytes = state_bytes(o->cfg.prec, rows > 0 ? rows : 1);
-    *m = *v = nullptr;
-    if (cudaMalloc(m, bytes) != cudaSuccess || cudaMalloc(v, bytes) != cudaSuccess) {
+    *m = nullptr;
+    if (cudaMalloc(m, state_bytes(o->cfg.prec, rows > 0 ? rows : 1)) != cudaSuccess) {
         cudaGetLastError();
-        cudaFree(*m);
-        cudaFree(*v);
-        *m = *v = nullptr;
+        *m = nullptr;
         return GS_ERR_OOM;
     }
     return GS_OK;
 }
 
-gs::StateView view_of(const gs_opt *o, void *m, void *v, int64_t capacity)
+gs::StateView view_of(const gs_opt *o, void *m, int64_t capacity)
 {
-    gs::StateView st{o->cfg.prec, m, v};
+    gs::StateView st{o->cfg.prec, m, static_cast<char *>(m) + state_row_bytes(o->cfg.prec)};
     if (o->cfg.prec == GS_MOM_FP8E4M3) {
         st.msc = fp8_scales(m, capacity);
-        st.vsc = fp8_scales(v, capacity);
+        st.vsc = st.msc + fp8_scale_floats(capacity);
     }
     return st;
 }
-gs::StateView view(const gs_opt *o) { return view_of(o, o->m, o->v, o->capacity); }
+gs::StateView view(const gs_opt *o) { return view_of(o, o->m, o->capacity); }
 
 // The optional terms of the extended step are not built for FP8 moments.
 bool terms_unsupported(const gs_opt *o, const gs_step_params *p)
@@ -256,10 +255,9 @@ void fill_args(const gs_opt *o, const gs_step_params *p, StepArgs *a)
 {
     memset(a, 0, sizeof(*a));
     a->m = o->m;
-    a->v = o->v;
     if (o->cfg.prec == GS_MOM_FP8E4M3) {
         a->msc = fp8_scales(o->m, o->capacity);
-        a->vsc = fp8_scales(o->v, o->capacity);
+        a->vsc = a->msc + fp8_scale_floats(o->capacity);
     }
     a->fac = o->fac;
     a->fac_len = o->tab_len;
@@ -375,7 +373,7 @@ gs_status gs_opt_init(gs_opt **out, const gs_opt_config *cfg, int64_t n_rows, vo
     }
     o->n_rows = n_rows;
     o->capacity = n_rows > 0 ? n_rows : 1;
-    st = alloc_state(o, o->capacity, &o->m, &o->v);
+    st = alloc_state(o, o->capacity, &o->m);
     if (st != GS_OK) {
         gs_opt_destroy(o);
         return st;
@@ -390,7 +388,7 @@ gs_status gs_opt_init(gs_opt **out, const gs_opt_config *cfg, int64_t n_rows, vo
         return GS_ERR_OOM;
     }
     const size_t sbytes = state_bytes(c.prec, o->capacity);
-    if ((e = cudaMemsetAsync(o->m, 0, sbytes, s)) != cudaSuccess || (e = cudaMemsetAsync(o->v, 0, sbytes, s)) != cudaSuccess ||
+    if ((e = cudaMemsetAsync(o->m, 0, sbytes, s)) != cudaSuccess ||
         (e = cudaMemsetAsync(o->err, 0, sizeof(int32_t), s)) != cudaSuccess ||
         (e = gs::launch_bias_table(c.beta1, c.beta2, o->tab_len, o->tab1, o->tab2, o->fac, s)) != cudaSuccess) {
         gs_opt_destroy(o);
@@ -412,9 +410,7 @@ void gs_opt_destroy(gs_opt *o)
     if (o->device >= 0) cudaSetDevice(o->device);
     cudaDeviceSynchronize();
     cudaFree(o->m);
-    cudaFree(o->v);
     cudaFree(o->m2);
-    cudaFree(o->v2);
     cudaFree(o->tab1);
     cudaFree(o->tab2);
     cudaFree(o->fac);
@@ -591,19 +587,17 @@ gs_status gs_reindex_state(gs_opt *o, const int32_t *src_rows, const uint8_t *re
         // the spare buffers are only read by the previous re-index, which
         // cudaFree waits for
         cudaFree(o->m2);
-        cudaFree(o->v2);
-        o->m2 = o->v2 = nullptr;
+        o->m2 = nullptr;
         o->capacity2 = 0;
         const int64_t cap = n_new > 0 ? n_new : 1;
-        gs_status a = alloc_state(o, cap, &o->m2, &o->v2);
+        gs_status a = alloc_state(o, cap, &o->m2);
         if (a != GS_OK) return a;
         o->capacity2 = cap;
     }
-    const gs::StateView out = view_of(o, o->m2, o->v2, o->capacity2);
+    const gs::StateView out = view_of(o, o->m2, o->capacity2);
     cudaError_t e = gs::launch_reindex(view(o), (int32_t)o->n_rows, out, (int32_t)n_new, src_rows, reset, o->err, s);
     if (e != cudaSuccess) return fail_cuda(o, e);
     std::swap(o->m, o->m2);
-    std::swap(o->v, o->v2);
     const int64_t tc = o->capacity;
     o->capacity = o->capacity2;
     o->capacity2 = tc;
@@ -636,7 +630,7 @@ gs_status gs_copy_rows(gs_opt *o, const gs_attrs *attrs, const gs_grads *grads, 
         return GS_ERR_INVALID_ARG;
     const int32_t row_bytes = (int32_t)state_row_bytes(o->cfg.prec);
     const int32_t used = o->cfg.prec == GS_MOM_FP32 ? 240 : row_bytes;    // FP32: 59 values + t
-    return fail_cuda(o, gs::launch_copy_rows(*attrs, *grads, o->m, o->v, row_bytes, used, rows, n_listed,
+    return fail_cuda(o, gs::launch_copy_rows(*attrs, *grads, o->m, row_bytes, used, rows, n_listed,
                                              (int32_t)n, o->err, static_cast<cudaStream_t>(stream)));
 }
 

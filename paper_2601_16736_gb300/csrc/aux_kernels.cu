@@ -177,11 +177,11 @@ __global__ void reindex_kernel(const StateView in, int32_t n_in, const StateView
     const bool fresh = s < 0 || (reset && reset[j]);
     uint4 mv = make_uint4(0u, 0u, 0u, 0u), vv = mv;
     if (!fresh) {      // each row is read once and written once: stream past L2
-        mv = __ldcs(reinterpret_cast<const uint4 *>(static_cast<const char *>(in.m) + (size_t)s * kRowBytes + 16 * c));
-        vv = __ldcs(reinterpret_cast<const uint4 *>(static_cast<const char *>(in.v) + (size_t)s * kRowBytes + 16 * c));
+        mv = __ldcs(reinterpret_cast<const uint4 *>(static_cast<const char *>(in.m) + (size_t)s * (2 * kRowBytes) + 16 * c));
+        vv = __ldcs(reinterpret_cast<const uint4 *>(static_cast<const char *>(in.v) + (size_t)s * (2 * kRowBytes) + 16 * c));
     }
-    __stcs(reinterpret_cast<uint4 *>(static_cast<char *>(out.m) + (size_t)j * kRowBytes + 16 * c), mv);
-    __stcs(reinterpret_cast<uint4 *>(static_cast<char *>(out.v) + (size_t)j * kRowBytes + 16 * c), vv);
+    __stcs(reinterpret_cast<uint4 *>(static_cast<char *>(out.m) + (size_t)j * (2 * kRowBytes) + 16 * c), mv);
+    __stcs(reinterpret_cast<uint4 *>(static_cast<char *>(out.v) + (size_t)j * (2 * kRowBytes) + 16 * c), vv);
 }
 
 // ------------------------------------------------------------ export/import
@@ -193,13 +193,13 @@ __global__ void reindex_kernel(const StateView in, int32_t n_in, const StateView
 __device__ __forceinline__ float *locate(const StateView &st, void *base, int64_t r, int c, __nv_bfloat16 **bf)
 {
     *bf = nullptr;
-    if (st.prec == GS_MOM_FP32) return static_cast<float *>(base) + r * kSlots + slot_of_col(c);
+    if (st.prec == GS_MOM_FP32) return static_cast<float *>(base) + r * (2 * kSlots) + slot_of_col(c);
     if (st.prec == GS_MOM_BF16) {
-        *bf = reinterpret_cast<__nv_bfloat16 *>(static_cast<char *>(base) + r * kRowBytesBf16) + slot_of_col(c);
+        *bf = reinterpret_cast<__nv_bfloat16 *>(static_cast<char *>(base) + r * (2 * kRowBytesBf16)) + slot_of_col(c);
         return nullptr;
     }
     // hybrid FP32 part: [0-2] SH DC, [3] t, [4-7] rot, [8-10] xyz, [11-13] scale, [14] opacity
-    char *row = static_cast<char *>(base) + r * kRowBytesHyb;
+    char *row = static_cast<char *>(base) + r * (2 * kRowBytesHyb);
     float *f = reinterpret_cast<float *>(row);
     if (c < 3) return f + 8 + c;
     if (c < 6) return f + 11 + (c - 3);
@@ -213,9 +213,9 @@ __device__ __forceinline__ float *locate(const StateView &st, void *base, int64_
 __device__ __forceinline__ uint32_t *t_of(const StateView &st, int64_t r)
 {
     char *m = static_cast<char *>(st.m);
-    if (st.prec == GS_MOM_FP32) return reinterpret_cast<uint32_t *>(m + r * kRowBytesF32 + kTByteF32);
-    if (st.prec == GS_MOM_BF16) return reinterpret_cast<uint32_t *>(m + r * kRowBytesBf16 + kTByteBf16);
-    return reinterpret_cast<uint32_t *>(m + r * kRowBytesHyb + kTByteHyb);
+    if (st.prec == GS_MOM_FP32) return reinterpret_cast<uint32_t *>(m + r * (2 * kRowBytesF32) + kTByteF32);
+    if (st.prec == GS_MOM_BF16) return reinterpret_cast<uint32_t *>(m + r * (2 * kRowBytesBf16) + kTByteBf16);
+    return reinterpret_cast<uint32_t *>(m + r * (2 * kRowBytesHyb) + kTByteHyb);
 }
 
 __global__ void export_kernel(const StateView st, int32_t n, float *__restrict__ m_out, float *__restrict__ v_out,
@@ -269,8 +269,8 @@ __global__ void export_f16b_kernel(const StateView st, int32_t n, float *__restr
     const int c = (int)(gid - r * kNumCols);
     int byte, group;
     f16b_slot(c, byte, group);
-    const char *mr = static_cast<const char *>(st.m) + r * kRowBytesF16B;
-    const char *vr = static_cast<const char *>(st.v) + r * kRowBytesF16B;
+    const char *mr = static_cast<const char *>(st.m) + r * (2 * kRowBytesF16B);
+    const char *vr = static_cast<const char *>(st.v) + r * (2 * kRowBytesF16B);
     if (m_out)
         m_out[gid] = __half2float(*reinterpret_cast<const __half *>(mr + byte)) * dec_scale((uint8_t)mr[kF16BExp + group]);
     if (v_out)
@@ -300,7 +300,7 @@ __global__ void import_f16b_kernel(const StateView st, int32_t n, const float *_
     for (int side = 0; side < 2; ++side) {
         const float *in = side ? v_in : m_in;
         if (!in) continue;
-        char *row = static_cast<char *>(side ? st.v : st.m) + r * kRowBytesF16B;
+        char *row = static_cast<char *>(side ? st.v : st.m) + r * (2 * kRowBytesF16B);
         float x[8];
         for (int q = 0; q < cnt; ++q) x[q] = in[r * kNumCols + cols[q]];
         const uint32_t e = group_exponent(x, cnt);
@@ -315,7 +315,7 @@ __global__ void import_f16b_kernel(const StateView st, int32_t n, const float *_
         row[kF16BExp + g] = (char)e;
     }
     if (t_in && g == 7)
-        *reinterpret_cast<uint16_t *>(static_cast<char *>(st.m) + r * kRowBytesF16B + kTByteF16B) =
+        *reinterpret_cast<uint16_t *>(static_cast<char *>(st.m) + r * (2 * kRowBytesF16B) + kTByteF16B) =
             (uint16_t)min(t_in[r], 65535u);
 }
 
@@ -409,8 +409,8 @@ __global__ void __launch_bounds__(kThreads) gather_small_kernel(const gs_attrs i
 struct CopyRowsArgs {
     gs_attrs a;
     gs_grads g;
-    char *m, *v;
-    int32_t row_bytes, chunks;              // state row stride; 16-B chunks used per row
+    char *m;
+    int32_t row_bytes, chunks;              // bytes of an m or v row; 16-B chunks used of each
     const int32_t *rows;
     int64_t nl;
     int32_t n;
@@ -465,7 +465,7 @@ __global__ void __launch_bounds__(kThreads) copy_rows_kernel(const CopyRowsArgs 
             const uint32_t b = grad_bits4(c.g.sh + r * 48 + 4 * i, c.zero);
             __stcs(t, xor4(*t, b));
         } else if (w < e_st) {
-            uint4 *t = reinterpret_cast<uint4 *>((w < e_m ? c.m : c.v) + r * c.row_bytes) + i;
+            uint4 *t = reinterpret_cast<uint4 *>(c.m + (2 * r + (w < e_m ? 0 : 1)) * c.row_bytes) + i;
             __stcs(t, *t);
         } else if (i == 1) {
             float4 *t = reinterpret_cast<float4 *>(c.a.rot + r * 4);
@@ -670,12 +670,12 @@ cudaError_t launch_gather_attrs(const gs_attrs &in, int32_t n_in, const gs_attrs
     return cudaGetLastError();
 }
 
-cudaError_t launch_copy_rows(const gs_attrs &a, const gs_grads &g, void *m, void *v, int32_t row_bytes,
+cudaError_t launch_copy_rows(const gs_attrs &a, const gs_grads &g, void *m, int32_t row_bytes,
                              int32_t used_bytes, const int32_t *rows, int64_t n_listed, int32_t n, int32_t *err,
                              cudaStream_t s)
 {
     if (n_listed <= 0) return cudaSuccess;
-    CopyRowsArgs c{a, g, static_cast<char *>(m), static_cast<char *>(v), row_bytes, used_bytes / 16, rows, n_listed,
+    CopyRowsArgs c{a, g, static_cast<char *>(m), row_bytes, used_bytes / 16, rows, n_listed,
                    n, err, 0u};
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);

@@ -90,7 +90,9 @@ struct Chunk {
 };
 
 // Every format provides
-//   kRowBytes, kTByte   row size and byte offset of t in the m row
+//   kRowBytes, kTByte   size of an m or v row (a state row holds both) and byte
+//                       offset of t in the m row
+//   row, vrow           the m and the v row of a primitive
 //   kTInSh              t is carried by SH item 0 (else by small chunk 14)
 //   load_sh / store_sh  the moments of SH columns kW*i .. kW*i+kW-1 (+ t)
 //   load_small / store_small  small chunk c in 12..14 (rotation; xyz +
@@ -104,14 +106,15 @@ struct State<GS_MOM_FP32> {
     static constexpr bool kTInSh = false;
     static __device__ __forceinline__ float *row(void *base, int32_t r)
     {
-        return static_cast<float *>(base) + (size_t)r * kSlots;
+        return static_cast<float *>(base) + (size_t)r * (2 * kSlots);
     }
+    static __device__ __forceinline__ float *vrow(void *base, int32_t r) { return row(base, r) + kSlots; }
     template <int kW>
     static __device__ __forceinline__ void load_sh(const StepArgs &a, int32_t r, int i, float *m, float *v, uint32_t &)
     {
 #pragma unroll
         for (int q = 0; q < kW / 4; ++q) {
-            const float4 x = ld4(row(a.m, r) + kW * i + 4 * q), y = ld4(row(a.v, r) + kW * i + 4 * q);
+            const float4 x = ld4(row(a.m, r) + kW * i + 4 * q), y = ld4(vrow(a.m, r) + kW * i + 4 * q);
             m[4 * q] = x.x; m[4 * q + 1] = x.y; m[4 * q + 2] = x.z; m[4 * q + 3] = x.w;
             v[4 * q] = y.x; v[4 * q + 1] = y.y; v[4 * q + 2] = y.z; v[4 * q + 3] = y.w;
         }
@@ -123,14 +126,14 @@ struct State<GS_MOM_FP32> {
 #pragma unroll
         for (int q = 0; q < kW / 4; ++q) {
             st4(row(a.m, r) + kW * i + 4 * q, make_float4(m[4 * q], m[4 * q + 1], m[4 * q + 2], m[4 * q + 3]));
-            st4(row(a.v, r) + kW * i + 4 * q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
+            st4(vrow(a.m, r) + kW * i + 4 * q, make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]));
         }
     }
     static __device__ __forceinline__ Chunk load_small(const StepArgs &a, int32_t r, int c)
     {
         Chunk k;
         k.m = ld4(row(a.m, r) + 4 * c);
-        k.v = ld4(row(a.v, r) + 4 * c);
+        k.v = ld4(vrow(a.m, r) + 4 * c);
         k.t = __float_as_uint(k.m.w);           // slot 59 of m (meaningful for c == 14)
         return k;
     }
@@ -138,7 +141,7 @@ struct State<GS_MOM_FP32> {
     {
         if (c == 14) k.m.w = __uint_as_float(k.t);
         st4(row(a.m, r) + 4 * c, k.m);
-        st4(row(a.v, r) + 4 * c, k.v);
+        st4(vrow(a.m, r) + 4 * c, k.v);
     }
 };
 
@@ -180,20 +183,21 @@ struct State<GS_MOM_BF16> {
     static constexpr bool kTInSh = false;
     static __device__ __forceinline__ char *row(void *base, int32_t r)
     {
-        return static_cast<char *>(base) + (size_t)r * kRowBytes;
+        return static_cast<char *>(base) + (size_t)r * (2 * kRowBytes);
     }
+    static __device__ __forceinline__ char *vrow(void *base, int32_t r) { return row(base, r) + kRowBytes; }
     template <int kW>
     static __device__ __forceinline__ void load_sh(const StepArgs &a, int32_t r, int i, float *m, float *v, uint32_t &)
     {
         load_bf16<kW>(row(a.m, r) + 2 * kW * i, m);
-        load_bf16<kW>(row(a.v, r) + 2 * kW * i, v);
+        load_bf16<kW>(vrow(a.m, r) + 2 * kW * i, v);
     }
     template <int kW>
     static __device__ __forceinline__ void store_sh(const StepArgs &a, int32_t r, int i, const float *m,
                                                     const float *v, uint32_t)
     {
         store_bf16_rn<kW>(row(a.m, r) + 2 * kW * i, m);
-        store_bf16_sr<kW>(row(a.v, r) + 2 * kW * i, v, a, r, kW * i);
+        store_bf16_sr<kW>(vrow(a.m, r) + 2 * kW * i, v, a, r, kW * i);
     }
     static __device__ __forceinline__ Chunk load_small(const StepArgs &a, int32_t r, int c)
     {
@@ -209,7 +213,7 @@ struct State<GS_MOM_BF16> {
             k.t = um.z;
         }
         k.m = make_float4(x[0], x[1], x[2], x[3]);
-        load_bf16<4>(row(a.v, r) + 8 * c, x);
+        load_bf16<4>(vrow(a.m, r) + 8 * c, x);
         k.v = make_float4(x[0], x[1], x[2], x[3]);
         return k;
     }
@@ -223,7 +227,7 @@ struct State<GS_MOM_BF16> {
                    make_uint4(pack_bf16x2(k.m.x, k.m.y), pack_bf16x2(k.m.z, k.m.w), k.t, 0u));
         }
         const float vv[4] = {k.v.x, k.v.y, k.v.z, k.v.w};
-        store_bf16_sr<4>(row(a.v, r) + 8 * c, vv, a, r, 4 * c);
+        store_bf16_sr<4>(vrow(a.m, r) + 8 * c, vv, a, r, 4 * c);
     }
 };
 
@@ -239,17 +243,18 @@ struct State<GS_MOM_BF16_HYBRID> {
     static constexpr bool kTInSh = true;
     static __device__ __forceinline__ char *row(void *base, int32_t r)
     {
-        return static_cast<char *>(base) + (size_t)r * kRowBytes;
+        return static_cast<char *>(base) + (size_t)r * (2 * kRowBytes);
     }
+    static __device__ __forceinline__ char *vrow(void *base, int32_t r) { return row(base, r) + kRowBytes; }
     template <int kW>
     static __device__ __forceinline__ void load_sh(const StepArgs &a, int32_t r, int i, float *m, float *v,
                                                    uint32_t &t)
     {
         load_bf16<kW>(row(a.m, r) + kHybShByte + 2 * kW * i, m);
-        load_bf16<kW>(row(a.v, r) + kHybShByte + 2 * kW * i, v);
+        load_bf16<kW>(vrow(a.m, r) + kHybShByte + 2 * kW * i, v);
         if (i == 0) {
             const float4 fm = *reinterpret_cast<const float4 *>(row(a.m, r));
-            const float4 fv = *reinterpret_cast<const float4 *>(row(a.v, r));
+            const float4 fv = *reinterpret_cast<const float4 *>(vrow(a.m, r));
             m[0] = fm.x; m[1] = fm.y; m[2] = fm.z;
             v[0] = fv.x; v[1] = fv.y; v[2] = fv.z;
             t = __float_as_uint(fm.w);
@@ -267,24 +272,24 @@ struct State<GS_MOM_BF16_HYBRID> {
         }
         if (i == 0) {
             st4(reinterpret_cast<float *>(row(a.m, r)), make_float4(m[0], m[1], m[2], __uint_as_float(t)));
-            st4(reinterpret_cast<float *>(row(a.v, r)), make_float4(v[0], v[1], v[2], 0.f));
+            st4(reinterpret_cast<float *>(vrow(a.m, r)), make_float4(v[0], v[1], v[2], 0.f));
             mm[0] = mm[1] = mm[2] = vv[0] = vv[1] = vv[2] = 0.f;   // BF16 DC slots are unused
         }
         store_bf16_rn<kW>(row(a.m, r) + kHybShByte + 2 * kW * i, mm);
-        store_bf16_sr<kW>(row(a.v, r) + kHybShByte + 2 * kW * i, vv, a, r, kW * i);
+        store_bf16_sr<kW>(vrow(a.m, r) + kHybShByte + 2 * kW * i, vv, a, r, kW * i);
     }
     static __device__ __forceinline__ Chunk load_small(const StepArgs &a, int32_t r, int c)
     {
         Chunk k;
         k.m = *reinterpret_cast<const float4 *>(row(a.m, r) + 16 * (c - 11));
-        k.v = *reinterpret_cast<const float4 *>(row(a.v, r) + 16 * (c - 11));
+        k.v = *reinterpret_cast<const float4 *>(vrow(a.m, r) + 16 * (c - 11));
         k.t = 0;
         return k;
     }
     static __device__ __forceinline__ void store_small(const StepArgs &a, int32_t r, int c, const Chunk &k)
     {
         st4(reinterpret_cast<float *>(row(a.m, r) + 16 * (c - 11)), k.m);
-        st4(reinterpret_cast<float *>(row(a.v, r) + 16 * (c - 11)), k.v);
+        st4(reinterpret_cast<float *>(vrow(a.m, r) + 16 * (c - 11)), k.v);
     }
 };
 
@@ -376,13 +381,14 @@ struct State<GS_MOM_FP16_BLOCK> {
     static constexpr bool kTInSh = false;
     static __device__ __forceinline__ char *row(void *base, int32_t r)
     {
-        return static_cast<char *>(base) + (size_t)r * kRowBytes;
+        return static_cast<char *>(base) + (size_t)r * (2 * kRowBytes);
     }
+    static __device__ __forceinline__ char *vrow(void *base, int32_t r) { return row(base, r) + kRowBytes; }
     template <int kW>
     static __device__ __forceinline__ void load_sh(const StepArgs &a, int32_t r, int i, float *m, float *v, uint32_t &)
     {
         static_assert(kW == 8, "FP16 block items cover 8 SH columns");
-        const char *mr = row(a.m, r), *vr = row(a.v, r);
+        const char *mr = row(a.m, r), *vr = vrow(a.m, r);
         const uint4 um = *reinterpret_cast<const uint4 *>(mr + 16 * i), uv = *reinterpret_cast<const uint4 *>(vr + 16 * i);
         const uint32_t wm[4] = {um.x, um.y, um.z, um.w}, wv[4] = {uv.x, uv.y, uv.z, uv.w};
         decode_w<8>(wm, dec_scale((uint8_t)mr[kF16BExp + i]), m);
@@ -392,7 +398,7 @@ struct State<GS_MOM_FP16_BLOCK> {
     static __device__ __forceinline__ void store_sh(const StepArgs &a, int32_t r, int i, const float *m,
                                                     const float *v, uint32_t)
     {
-        char *mr = row(a.m, r), *vr = row(a.v, r);
+        char *mr = row(a.m, r), *vr = vrow(a.m, r);
         uint32_t wm[4], wv[4];
         const uint32_t em = encode_rn_w<8>(m, wm), ev = encode_sr_w<8>(v, wv, a, r, 11 + 8 * i);
         __stcs(reinterpret_cast<uint4 *>(mr + 16 * i), make_uint4(wm[0], wm[1], wm[2], wm[3]));
@@ -413,7 +419,7 @@ __device__ __forceinline__ bool small_item_f16b(const StepArgs &a, const int32_t
                                                 const float2 f, const float3 nz)
 {
     using S = State<GS_MOM_FP16_BLOCK>;
-    char *mr = S::row(a.m, row), *vr = S::row(a.v, row);
+    char *mr = S::row(a.m, row), *vr = S::vrow(a.m, row);
     const size_t r = (size_t)row;
     if (c == 12) {
         const uint2 um = *reinterpret_cast<const uint2 *>(mr + kF16BRot), uv = *reinterpret_cast<const uint2 *>(vr + kF16BRot);
@@ -495,7 +501,7 @@ __device__ __forceinline__ bool small_item_f16b(const StepArgs &a, const int32_t
 __device__ __forceinline__ void rsr_small_f16b(const StepArgs &a, const int32_t row, const int c)
 {
     using S = State<GS_MOM_FP16_BLOCK>;
-    char *mr = S::row(a.m, row), *vr = S::row(a.v, row);
+    char *mr = S::row(a.m, row), *vr = S::vrow(a.m, row);
     if (c == 12) {
         const uint2 um = *reinterpret_cast<const uint2 *>(mr + kF16BRot), uv = *reinterpret_cast<const uint2 *>(vr + kF16BRot);
         const uint32_t wm[2] = {um.x, um.y}, wv[2] = {uv.x, uv.y};
@@ -525,7 +531,7 @@ __device__ __forceinline__ void rsr_small_f16b(const StepArgs &a, const int32_t 
 }
 
 // Ask L2 to fetch the contiguous parts a visible row's items will read (SH
-// attributes and gradients, m and v rows; cp.async.bulk.prefetch.L2), as
+// attributes and gradients, the state row; cp.async.bulk.prefetch.L2), as
 // soon as the row is known to be visible.  Worth it for sparse tiles: their
 // rows are scattered, and the items' later loads then hit L2.  Dense tiles
 // already stream well and only pay for the extra requests, so callers skip
@@ -536,10 +542,8 @@ __device__ __forceinline__ void prefetch_row_l2(const StepArgs &a, int32_t row)
     const size_t r = (size_t)row;
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], 192;" ::"l"(a.a_sh + r * 48) : "memory");
     if (!a.g_host) asm volatile("cp.async.bulk.prefetch.L2.global [%0], 192;" ::"l"(a.g_sh + r * 48) : "memory");
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(static_cast<const char *>(a.m) + r * kRowBytes),
-                 "n"(kRowBytes) : "memory");
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(static_cast<const char *>(a.v) + r * kRowBytes),
-                 "n"(kRowBytes) : "memory");
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(static_cast<const char *>(a.m) + r * (2 * kRowBytes)),
+                 "n"(2 * kRowBytes) : "memory");
 }
 
 // Ask L2 for the visibility inputs (means or mask bytes) of the tile one wave

@@ -74,7 +74,7 @@ __device__ __forceinline__ bool small_item_x_f16b(const StepArgs &a, const int32
 {
     using S = State<GS_MOM_FP16_BLOCK>;
     const bool aiu = !vis && (fl & kFAiu);
-    char *mr = S::row(a.m, row), *vr = S::row(a.v, row);
+    char *mr = S::row(a.m, row), *vr = S::vrow(a.m, row);
     const size_t r = (size_t)row;
     if (c == 12) {
         const uint2 um = *reinterpret_cast<const uint2 *>(mr + kF16BRot), uv = *reinterpret_cast<const uint2 *>(vr + kF16BRot);
@@ -328,7 +328,7 @@ __device__ __forceinline__ void tile_decide_x(const StepArgs &a, const int vis_s
             if (a.noise == GS_NOISE_ALL || (a.noise == GS_NOISE_VISIBLE && vis)) fl |= kFNoise;
             const bool aiu_draw = a.aiu && !vis && aiu_sampled(a, (int32_t)row);
             if ((vis || aiu_draw) && !a.bias_mode) {
-                const char *tp = static_cast<const char *>(a.m) + (size_t)row * kRowBytes + kTByte;
+                const char *tp = static_cast<const char *>(a.m) + (size_t)row * (2 * kRowBytes) + kTByte;
                 if constexpr (kTByte % 4 == 0) t_old[j] = *reinterpret_cast<const uint32_t *>(tp);
                 else t_old[j] = *reinterpret_cast<const uint16_t *>(tp);      // FP16-block rows: uint16 t
             }

@@ -1,6 +1,6 @@
 // FP8 (e4m3) moments with per-256-row block scales.
 //
-// Storage: m and v rows of 64 bytes, the 59 e4m3 codes in work-chunk order
+// Storage: m and v rows of 64 bytes side by side (one 128-B line a primitive), the 59 e4m3 codes in work-chunk order
 // (SH 0-47, rotation 48-51, xyz 52-54, opacity 55, scale 56-58; byte 59 is
 // padding and bytes 60-63 of the m row hold the step counter t), so that
 // each 4-value work chunk is one 32-bit word; and for every block of 256
@@ -42,6 +42,7 @@ namespace {
 constexpr int kF8Tile = 256;                 // rows per block scale = rows per CTA
 constexpr int kF8Cols = 59;
 constexpr int kF8Row = 64;                   // bytes per code row
+constexpr int kF8Step = 2 * kF8Row;          // from a primitive's m (or v) row to the next one's
 constexpr int kF8TWord = 15;                 // 32-bit word of the m row holding t
 constexpr int kF8MinBlocks = 4;
 // A block recomputes its scales from all of its rows (and may shrink them)
@@ -252,7 +253,7 @@ __device__ __forceinline__ void f8_block_grow(const StepArgs &a, const int vis_s
 {
     const int tid = threadIdx.x, lane = tid & 31;
     const int64_t r0 = (int64_t)tile * kF8Tile;
-    uint8_t *gm = static_cast<uint8_t *>(a.m), *gv = static_cast<uint8_t *>(a.v);
+    uint8_t *gm = static_cast<uint8_t *>(a.m), *gv = gm + kF8Row;
     if (tid < 64) {
         const float sm = tid < kF8Cols ? a.msc[tile * 64 + tid] : 0.f;
         const float sv = tid < kF8Cols ? a.vsc[tile * 64 + tid] : 0.f;
@@ -276,7 +277,7 @@ __device__ __forceinline__ void f8_block_grow(const StepArgs &a, const int vis_s
         } else {
             vis = true;
         }
-        if (vis) t_old = reinterpret_cast<const uint32_t *>(gm + row * kF8Row)[kF8TWord];
+        if (vis) t_old = reinterpret_cast<const uint32_t *>(gm + row * kF8Step)[kF8TWord];
         if (a.mask_out) a.mask_out[row] = vis ? 1 : 0;
         if (a.restate) smp = stss_sampled(a, (int32_t)row);
     }
@@ -304,8 +305,8 @@ __device__ __forceinline__ void f8_block_grow(const StepArgs &a, const int vis_s
         const int64_t r = r0 + lr;
         float th[4], g[4], m[4], v[4];
         if (fl & 1) f8_load_chunk(a, r, k, th, g);
-        uint32_t *pm = reinterpret_cast<uint32_t *>(gm + r * kF8Row) + k;
-        uint32_t *pv = reinterpret_cast<uint32_t *>(gv + r * kF8Row) + k;
+        uint32_t *pm = reinterpret_cast<uint32_t *>(gm + r * kF8Step) + k;
+        uint32_t *pv = reinterpret_cast<uint32_t *>(gv + r * kF8Step) + k;
         f8_dec4(*pm, &S.s_old[0][4 * k], m);
         f8_dec4(*pv, &S.s_old[1][4 * k], v);
         f8_apply_chunk(a, k, fl & 1, fl & 2, S.fac[lr], th, g, m, v);
@@ -348,7 +349,7 @@ __device__ __forceinline__ void f8_block_grow(const StepArgs &a, const int vis_s
     for (int idx = tid; idx < nrow * nmov; idx += kThreads) {
         const int lr = idx / nmov, q = S.mov[idx - lr * nmov], w = q >> 6, c = q & 63;
         if ((S.dmask[lr] >> (c >> 2)) & 1u) continue;
-        uint8_t *pb = (w ? gv : gm) + (r0 + lr) * kF8Row + c;
+        uint8_t *pb = (w ? gv : gm) + (r0 + lr) * kF8Step + c;
         const float x = f8_dec(*pb) * S.s_old[w][c] * S.s_inv[w][c];
         *pb = (uint8_t)(w ? f8_rn_floor(x) : f8_rn(x));
     }
@@ -360,8 +361,8 @@ __device__ __forceinline__ void f8_block_grow(const StepArgs &a, const int vis_s
         const int64_t r = r0 + lr;
         float th[4], g[4], m[4], v[4];
         if (fl & 1) f8_load_chunk(a, r, k, th, g);
-        uint32_t *pm = reinterpret_cast<uint32_t *>(gm + r * kF8Row) + k;
-        uint32_t *pv = reinterpret_cast<uint32_t *>(gv + r * kF8Row) + k;
+        uint32_t *pm = reinterpret_cast<uint32_t *>(gm + r * kF8Step) + k;
+        uint32_t *pv = reinterpret_cast<uint32_t *>(gv + r * kF8Step) + k;
         f8_dec4(*pm, &S.s_old[0][4 * k], m);
         f8_dec4(*pv, &S.s_old[1][4 * k], v);
         f8_apply_chunk(a, k, fl & 1, fl & 2, S.fac[lr], th, g, m, v);
@@ -370,7 +371,7 @@ __device__ __forceinline__ void f8_block_grow(const StepArgs &a, const int vis_s
         __stcs(pm, f8_enc4_rn(m, &S.s_inv[0][4 * k]));
         __stcs(pv, f8_enc4_sr(v, &S.s_inv[1][4 * k], f8_rnd(a, r, k)));
     }
-    if (tid < nrow && vis) reinterpret_cast<uint32_t *>(gm + row * kF8Row)[kF8TWord] = t_old + 1u;   // Sec. 3.2
+    if (tid < nrow && vis) reinterpret_cast<uint32_t *>(gm + row * kF8Step)[kF8TWord] = t_old + 1u;   // Sec. 3.2
 }
 
 // Shared arrays of a block on its full pass.
@@ -421,11 +422,11 @@ __device__ __forceinline__ void f8_block_full(const StepArgs &a, const int vis_s
     const int64_t r0 = (int64_t)tile * kF8Tile;
     const int nrow = (int)min((int64_t)kF8Tile, (int64_t)a.n_rows - r0);
 
-    const uint4 *gm = reinterpret_cast<const uint4 *>(static_cast<const char *>(a.m) + r0 * kF8Row);
-    const uint4 *gv = reinterpret_cast<const uint4 *>(static_cast<const char *>(a.v) + r0 * kF8Row);
-    for (int q = tid; q < nrow * (kF8Row / 16); q += kThreads) {
-        reinterpret_cast<uint4 *>(cm)[q] = __ldcs(gm + q);
-        reinterpret_cast<uint4 *>(cv)[q] = __ldcs(gv + q);
+    uint4 *gs4 = reinterpret_cast<uint4 *>(static_cast<char *>(a.m) + r0 * kF8Step);
+    constexpr int kCh = kF8Row / 16;          // 16-B chunks of an m or v row
+    for (int q = tid; q < nrow * 2 * kCh; q += kThreads) {
+        const int lr = q / (2 * kCh), c = q % (2 * kCh);
+        reinterpret_cast<uint4 *>(c < kCh ? cm : cv)[lr * kCh + c % kCh] = __ldcs(gs4 + q);
     }
     if (tid < 64) {
         s_old[0][tid] = tid < kF8Cols ? a.msc[tile * 64 + tid] : 0.f;
@@ -578,13 +579,11 @@ __device__ __forceinline__ void f8_block_full(const StepArgs &a, const int vis_s
     if (tid < nrow && vis) cm[tid * (kF8Row / 4) + kF8TWord] += 1u;   // the row's own step count (Sec. 3.2)
     __syncthreads();
     // write back the rows that changed: all of them when a scale moved
-    uint4 *om4 = reinterpret_cast<uint4 *>(static_cast<char *>(a.m) + r0 * kF8Row);
-    uint4 *ov4 = reinterpret_cast<uint4 *>(static_cast<char *>(a.v) + r0 * kF8Row);
     const bool all = s_moved != 0;
-    for (int q = tid; q < nrow * (kF8Row / 16); q += kThreads) {
-        if (!all && !flg[q / (kF8Row / 16)]) continue;
-        __stcs(om4 + q, reinterpret_cast<const uint4 *>(cm)[q]);
-        __stcs(ov4 + q, reinterpret_cast<const uint4 *>(cv)[q]);
+    for (int q = tid; q < nrow * 2 * kCh; q += kThreads) {
+        const int lr = q / (2 * kCh), c = q % (2 * kCh);
+        if (!all && !flg[lr]) continue;
+        __stcs(gs4 + q, reinterpret_cast<const uint4 *>(c < kCh ? cm : cv)[lr * kCh + c % kCh]);
     }
 }
 
@@ -622,9 +621,9 @@ __global__ void export_fp8_kernel(const uint8_t *__restrict__ m, const uint8_t *
     const int64_t r = idx / kF8Cols;
     const int c = f8_slot((int)(idx - r * kF8Cols));
     const int64_t sb = (r / kF8Tile) * 64 + c;
-    if (m_out) m_out[idx] = f8_dec(m[r * kF8Row + c]) * msc[sb];
-    if (v_out) v_out[idx] = f8_dec(v[r * kF8Row + c]) * vsc[sb];
-    if (t_out && c == 0) t_out[r] = reinterpret_cast<const uint32_t *>(m + r * kF8Row)[kF8TWord];
+    if (m_out) m_out[idx] = f8_dec(m[r * kF8Step + c]) * msc[sb];
+    if (v_out) v_out[idx] = f8_dec(v[r * kF8Step + c]) * vsc[sb];
+    if (t_out && c == 0) t_out[r] = reinterpret_cast<const uint32_t *>(m + r * kF8Step)[kF8TWord];
 }
 
 // One CTA per block: the slot maxima of the imported values, the scales,
@@ -662,10 +661,10 @@ __global__ void __launch_bounds__(kThreads) import_fp8_kernel(uint8_t *__restric
     __syncthreads();
     for (int q = tid; q < nrow * kF8Cols; q += kThreads) {
         const int lr = q / kF8Cols, c = f8_slot(q - lr * kF8Cols);
-        if (m_in) m[(r0 + lr) * kF8Row + c] = (uint8_t)f8_rn(m_in[e0 + q] * s_inv[0][c]);
-        if (v_in) v[(r0 + lr) * kF8Row + c] = (uint8_t)f8_rn_floor(v_in[e0 + q] * s_inv[1][c]);
+        if (m_in) m[(r0 + lr) * kF8Step + c] = (uint8_t)f8_rn(m_in[e0 + q] * s_inv[0][c]);
+        if (v_in) v[(r0 + lr) * kF8Step + c] = (uint8_t)f8_rn_floor(v_in[e0 + q] * s_inv[1][c]);
     }
-    if (t_in && tid < nrow) reinterpret_cast<uint32_t *>(m + (r0 + tid) * kF8Row)[kF8TWord] = t_in[r0 + tid];
+    if (t_in && tid < nrow) reinterpret_cast<uint32_t *>(m + (r0 + tid) * kF8Step)[kF8TWord] = t_in[r0 + tid];
 }
 
 // ------------------------------------------------------------- re-index
@@ -703,8 +702,8 @@ __global__ void __launch_bounds__(kThreads) reindex_fp8_kernel(
         const int64_t s = s_src[lr];
         if (s < 0) continue;
         const int64_t sb = (s / kF8Tile) * 64 + c;
-        atomicMax(&s_max[0][c], __float_as_uint(fabsf(f8_dec(m_in[s * kF8Row + c]) * msc_in[sb])));
-        atomicMax(&s_max[1][c], __float_as_uint(fabsf(f8_dec(v_in[s * kF8Row + c]) * vsc_in[sb])));
+        atomicMax(&s_max[0][c], __float_as_uint(fabsf(f8_dec(m_in[s * kF8Step + c]) * msc_in[sb])));
+        atomicMax(&s_max[1][c], __float_as_uint(fabsf(f8_dec(v_in[s * kF8Step + c]) * vsc_in[sb])));
     }
     __syncthreads();
     if (tid < 2 * kF8Cols) {
@@ -721,20 +720,20 @@ __global__ void __launch_bounds__(kThreads) reindex_fp8_kernel(
         uint32_t cmv = 0u, cvv = 0u;
         if (s >= 0) {
             const int64_t sb = (s / kF8Tile) * 64 + c;
-            cmv = f8_rn(f8_dec(m_in[s * kF8Row + c]) * msc_in[sb] * s_inv[0][c]);
-            cvv = f8_rn_floor(f8_dec(v_in[s * kF8Row + c]) * vsc_in[sb] * s_inv[1][c]);
+            cmv = f8_rn(f8_dec(m_in[s * kF8Step + c]) * msc_in[sb] * s_inv[0][c]);
+            cvv = f8_rn_floor(f8_dec(v_in[s * kF8Step + c]) * vsc_in[sb] * s_inv[1][c]);
         }
-        m_out[(r0 + lr) * kF8Row + c] = (uint8_t)cmv;
-        v_out[(r0 + lr) * kF8Row + c] = (uint8_t)cvv;
+        m_out[(r0 + lr) * kF8Step + c] = (uint8_t)cmv;
+        v_out[(r0 + lr) * kF8Step + c] = (uint8_t)cvv;
     }
     if (tid < nrow) {
         const int64_t s = s_src[tid];
-        const uint32_t t = s >= 0 ? reinterpret_cast<const uint32_t *>(m_in + s * kF8Row)[kF8TWord] : 0u;
-        uint32_t *mo = reinterpret_cast<uint32_t *>(m_out + (r0 + tid) * kF8Row);
+        const uint32_t t = s >= 0 ? reinterpret_cast<const uint32_t *>(m_in + s * kF8Step)[kF8TWord] : 0u;
+        uint32_t *mo = reinterpret_cast<uint32_t *>(m_out + (r0 + tid) * kF8Step);
         mo[kF8TWord] = t;
-        reinterpret_cast<uint32_t *>(v_out + (r0 + tid) * kF8Row)[kF8TWord] = 0u;
-        m_out[(r0 + tid) * kF8Row + 59] = 0;
-        v_out[(r0 + tid) * kF8Row + 59] = 0;
+        reinterpret_cast<uint32_t *>(v_out + (r0 + tid) * kF8Step)[kF8TWord] = 0u;
+        m_out[(r0 + tid) * kF8Step + 59] = 0;
+        v_out[(r0 + tid) * kF8Step + 59] = 0;
     }
 }
 

@@ -89,7 +89,7 @@ __device__ __forceinline__ void tile_decide(const StepArgs &a, const int vis_src
                 vis = true;
             }
             if (vis && !a.bias_mode) {
-                const char *tp = static_cast<const char *>(a.m) + (size_t)row * kRowBytes + kTByte;
+                const char *tp = static_cast<const char *>(a.m) + (size_t)row * (2 * kRowBytes) + kTByte;
                 if constexpr (kTByte % 4 == 0) t_old[j] = *reinterpret_cast<const uint32_t *>(tp);
                 else t_old[j] = *reinterpret_cast<const uint16_t *>(tp);      // FP16-block rows: uint16 t
             }
