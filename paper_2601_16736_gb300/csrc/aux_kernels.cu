@@ -1,7 +1,7 @@
 // Kernels around the fused step: the standalone visibility filter with
 // global compaction, the FP64 bias-correction table, optimizer-state
-// re-indexing across row-set changes, canonical-layout export/import, and
-// the attribute gather that accompanies a re-index.
+// re-indexing across row-set changes, and the attribute gather that
+// accompanies a re-index.
 
 #include <algorithm>
 
@@ -182,141 +182,6 @@ __global__ void reindex_kernel(const StateView in, int32_t n_in, const StateView
     }
     __stcs(reinterpret_cast<uint4 *>(static_cast<char *>(out.m) + (size_t)j * (2 * kRowBytes) + 16 * c), mv);
     __stcs(reinterpret_cast<uint4 *>(static_cast<char *>(out.v) + (size_t)j * (2 * kRowBytes) + 16 * c), vv);
-}
-
-// ------------------------------------------------------------ export/import
-// Canonical layout: [n][59] FP32 in the column order xyz, scale, rot,
-// opacity, sh; one thread per (row, column).
-
-// Where column c of row r of one moment array lives: a pointer to an FP32
-// value, or (through *bf) to a BF16 value.
-__device__ __forceinline__ float *locate(const StateView &st, void *base, int64_t r, int c, __nv_bfloat16 **bf)
-{
-    *bf = nullptr;
-    if (st.prec == GS_MOM_FP32) return static_cast<float *>(base) + r * (2 * kSlots) + slot_of_col(c);
-    if (st.prec == GS_MOM_BF16) {
-        *bf = reinterpret_cast<__nv_bfloat16 *>(static_cast<char *>(base) + r * (2 * kRowBytesBf16)) + slot_of_col(c);
-        return nullptr;
-    }
-    // hybrid FP32 part: [0-2] SH DC, [3] t, [4-7] rot, [8-10] xyz, [11-13] scale, [14] opacity
-    char *row = static_cast<char *>(base) + r * (2 * kRowBytesHyb);
-    float *f = reinterpret_cast<float *>(row);
-    if (c < 3) return f + 8 + c;
-    if (c < 6) return f + 11 + (c - 3);
-    if (c < 10) return f + 4 + (c - 6);
-    if (c == 10) return f + 14;
-    if (c < 14) return f + (c - 11);
-    *bf = reinterpret_cast<__nv_bfloat16 *>(row + kHybShByte) + (c - 11);
-    return nullptr;
-}
-
-__device__ __forceinline__ uint32_t *t_of(const StateView &st, int64_t r)
-{
-    char *m = static_cast<char *>(st.m);
-    if (st.prec == GS_MOM_FP32) return reinterpret_cast<uint32_t *>(m + r * (2 * kRowBytesF32) + kTByteF32);
-    if (st.prec == GS_MOM_BF16) return reinterpret_cast<uint32_t *>(m + r * (2 * kRowBytesBf16) + kTByteBf16);
-    return reinterpret_cast<uint32_t *>(m + r * (2 * kRowBytesHyb) + kTByteHyb);
-}
-
-__global__ void export_kernel(const StateView st, int32_t n, float *__restrict__ m_out, float *__restrict__ v_out,
-                              uint32_t *__restrict__ t_out)
-{
-    const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= (int64_t)n * kNumCols) return;
-    const int64_t r = gid / kNumCols;
-    const int c = (int)(gid - r * kNumCols);
-    __nv_bfloat16 *b;
-    if (m_out) {
-        const float *p = locate(st, st.m, r, c, &b);
-        m_out[gid] = p ? *p : __bfloat162float(*b);
-    }
-    if (v_out) {
-        const float *p = locate(st, st.v, r, c, &b);
-        v_out[gid] = p ? *p : __bfloat162float(*b);
-    }
-    if (t_out && c == 0) t_out[r] = *t_of(st, r);
-}
-
-__global__ void import_kernel(const StateView st, int32_t n, const float *__restrict__ m_in,
-                              const float *__restrict__ v_in, const uint32_t *__restrict__ t_in)
-{
-    const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= (int64_t)n * kNumCols) return;
-    const int64_t r = gid / kNumCols;
-    const int c = (int)(gid - r * kNumCols);
-    __nv_bfloat16 *b;
-    if (m_in) {
-        float *p = locate(st, st.m, r, c, &b);
-        if (p) *p = m_in[gid]; else *b = __float2bfloat16_rn(m_in[gid]);
-    }
-    if (v_in) {
-        float *p = locate(st, st.v, r, c, &b);
-        if (p) *p = v_in[gid]; else *b = __float2bfloat16_rn(v_in[gid]);
-    }
-    if (t_in && c == 0) *t_of(st, r) = t_in[r];
-}
-
-// FP16-block rows: export decodes one value per thread (its group exponent
-// beside it); import encodes one group per thread (8 SH columns, rotation,
-// xyz + scale + opacity) so that the group's shared exponent can be chosen,
-// rounding to nearest.  t is a uint16 at kTByteF16B (saturated on import).
-__global__ void export_f16b_kernel(const StateView st, int32_t n, float *__restrict__ m_out,
-                                   float *__restrict__ v_out, uint32_t *__restrict__ t_out)
-{
-    const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= (int64_t)n * kNumCols) return;
-    const int64_t r = gid / kNumCols;
-    const int c = (int)(gid - r * kNumCols);
-    int byte, group;
-    f16b_slot(c, byte, group);
-    const char *mr = static_cast<const char *>(st.m) + r * (2 * kRowBytesF16B);
-    const char *vr = static_cast<const char *>(st.v) + r * (2 * kRowBytesF16B);
-    if (m_out)
-        m_out[gid] = __half2float(*reinterpret_cast<const __half *>(mr + byte)) * dec_scale((uint8_t)mr[kF16BExp + group]);
-    if (v_out)
-        v_out[gid] = __half2float(*reinterpret_cast<const __half *>(vr + byte)) * dec_scale((uint8_t)vr[kF16BExp + group]);
-    if (t_out && c == 0) t_out[r] = *reinterpret_cast<const uint16_t *>(mr + kTByteF16B);
-}
-
-__global__ void import_f16b_kernel(const StateView st, int32_t n, const float *__restrict__ m_in,
-                                   const float *__restrict__ v_in, const uint32_t *__restrict__ t_in)
-{
-    const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (gid >= (int64_t)n * 8) return;
-    const int64_t r = gid / 8;
-    const int g = (int)(gid - r * 8);
-    int cols[8], cnt;
-    if (g < 6) {
-        cnt = 8;
-        for (int q = 0; q < 8; ++q) cols[q] = 11 + 8 * g + q;
-    } else if (g == 6) {
-        cnt = 4;
-        for (int q = 0; q < 4; ++q) cols[q] = 6 + q;
-    } else {
-        cnt = 7;
-        for (int q = 0; q < 6; ++q) cols[q] = q;
-        cols[6] = 10;
-    }
-    for (int side = 0; side < 2; ++side) {
-        const float *in = side ? v_in : m_in;
-        if (!in) continue;
-        char *row = static_cast<char *>(side ? st.v : st.m) + r * (2 * kRowBytesF16B);
-        float x[8];
-        for (int q = 0; q < cnt; ++q) x[q] = in[r * kNumCols + cols[q]];
-        const uint32_t e = group_exponent(x, cnt);
-        const float sc = e ? enc_scale(e) : 0.f;
-        for (int q = 0; q < cnt; ++q) {
-            int byte, group;
-            f16b_slot(cols[q], byte, group);
-            uint32_t h = e ? h_bits(x[q] * sc) : 0u;
-            if (side && (h & 0x7fffu) == 0u && x[q] > 0.f) h = 1u;     // a positive v stays positive
-            *reinterpret_cast<uint16_t *>(row + byte) = (uint16_t)h;
-        }
-        row[kF16BExp + g] = (char)e;
-    }
-    if (t_in && g == 7)
-        *reinterpret_cast<uint16_t *>(static_cast<char *>(st.m) + r * (2 * kRowBytesF16B) + kTByteF16B) =
-            (uint16_t)min(t_in[r], 65535u);
 }
 
 // ----------------------------------------------------------- attribute gather
@@ -630,30 +495,6 @@ cudaError_t launch_reindex(const StateView &in, int32_t n_in, const StateView &o
     default:
         return cudaErrorNotSupported;
     }
-    return cudaGetLastError();
-}
-
-cudaError_t launch_export(const StateView &st, int32_t n, float *m_out, float *v_out, uint32_t *t_out,
-                          cudaStream_t s)
-{
-    if (n <= 0) return cudaSuccess;
-    if (st.prec == GS_MOM_FP8E4M3) return launch_export_fp8(st, n, m_out, v_out, t_out, s);
-    if (st.prec == GS_MOM_FP16_BLOCK)
-        export_f16b_kernel<<<blocks_for((int64_t)n * kNumCols), kThreads, 0, s>>>(st, n, m_out, v_out, t_out);
-    else
-        export_kernel<<<blocks_for((int64_t)n * kNumCols), kThreads, 0, s>>>(st, n, m_out, v_out, t_out);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_import(const StateView &st, int32_t n, const float *m_in, const float *v_in,
-                          const uint32_t *t_in, cudaStream_t s)
-{
-    if (n <= 0) return cudaSuccess;
-    if (st.prec == GS_MOM_FP8E4M3) return launch_import_fp8(st, n, m_in, v_in, t_in, s);
-    if (st.prec == GS_MOM_FP16_BLOCK)
-        import_f16b_kernel<<<blocks_for((int64_t)n * 8), kThreads, 0, s>>>(st, n, m_in, v_in, t_in);
-    else
-        import_kernel<<<blocks_for((int64_t)n * kNumCols), kThreads, 0, s>>>(st, n, m_in, v_in, t_in);
     return cudaGetLastError();
 }
 

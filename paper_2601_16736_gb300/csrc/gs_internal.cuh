@@ -48,19 +48,7 @@ constexpr int kRowBytesHyb = 160, kTByteHyb = 12, kHybShByte = 64;
 // columns at 16i), the 8 item exponents at 96 + item, rotation at 104,
 // xyz / scale / opacity at 112 .. 125, t (uint16) at 126.
 constexpr int kRowBytesF16B = 128, kTByteF16B = 126, kF16BExp = 96, kF16BRot = 104, kF16BXso = 112;
-constexpr int kSlotSh = 0, kSlotRot = 48, kSlotXyz = 52, kSlotScale = 55, kSlotOpacity = 58;
-constexpr int kSlotT = 59;
 constexpr int kNumCols = 59;
-
-// canonical column (xyz, scale, rot, opacity, sh) -> state slot
-__host__ __device__ inline int slot_of_col(int c)
-{
-    if (c < 3) return kSlotXyz + c;
-    if (c < 6) return kSlotScale + (c - 3);
-    if (c < 10) return kSlotRot + (c - 6);
-    if (c == 10) return kSlotOpacity;
-    return kSlotSh + (c - 11);
-}
 
 enum VisSource : int { kVisAll = 0, kVisMask = 1, kVisCamera = 2 };
 
@@ -270,19 +258,6 @@ __device__ __forceinline__ uint32_t group_exponent(const float *x, int n)
 // 2^(141 - e) and 2^(e - 141) as exact FP32 powers of two (15 <= e <= 254)
 __device__ __forceinline__ float enc_scale(uint32_t e) { return __uint_as_float((268u - e) << 23); }
 __device__ __forceinline__ float dec_scale(uint32_t e) { return e ? __uint_as_float((e - 14u) << 23) : 0.f; }
-
-__device__ __forceinline__ uint32_t h_bits(float y) { return __half_as_ushort(__float2half_rn(y)); }
-
-
-// Canonical column c -> byte offset of its FP16 value in an FP16-block row
-// and the index of its group exponent.
-__host__ __device__ inline void f16b_slot(int c, int &byte, int &group)
-{
-    if (c < 6) { byte = kF16BXso + 2 * c; group = 7; }                  // xyz, scale
-    else if (c < 10) { byte = kF16BRot + 2 * (c - 6); group = 6; }      // rotation
-    else if (c == 10) { byte = kF16BXso + 12; group = 7; }              // opacity
-    else { byte = 2 * (c - 11); group = (c - 11) / 8; }                 // SH
-}
 
 // Scene table of one batched launch (in device memory, written by one
 // host-to-device copy before each launch or graph replay).

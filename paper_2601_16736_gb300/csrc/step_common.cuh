@@ -22,6 +22,37 @@ __device__ __forceinline__ float4 ldg4_stream(const float *p)
 // results are not read again in this step: store them evict-first
 __device__ __forceinline__ void st4(float *p, float4 x) { __stcs(reinterpret_cast<float4 *>(p), x); }
 
+// Asynchronous copies from device to shared memory: a CTA keeps a whole tile in
+// flight without holding it in registers.
+__device__ __forceinline__ void cp_async16(void *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async4(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// nf consecutive canonical floats between device and shared memory, by the
+// whole CTA: float4 where the caller's array is 16-B aligned, else floats
+// (the entry points ask for 4-B alignment only).  The load is asynchronous
+// (cp_async_wait and a barrier before use).
+__device__ __forceinline__ void load_canonical(const float *__restrict__ in, int nf, float *xs)
+{
+    const int nv = ((uintptr_t)in & 15u) ? 0 : nf / 4;
+    for (int q = threadIdx.x; q < nv; q += kThreads) cp_async16(xs + 4 * q, in + 4 * q);
+    for (int q = 4 * nv + threadIdx.x; q < nf; q += kThreads) cp_async4(xs + q, in + q);
+}
+__device__ __forceinline__ void store_canonical(float *__restrict__ out, int nf, const float *xs)
+{
+    const int nv = ((uintptr_t)out & 15u) ? 0 : nf / 4;
+    for (int q = threadIdx.x; q < nv; q += kThreads) st4(out + 4 * q, *reinterpret_cast<const float4 *>(xs + 4 * q));
+    for (int q = 4 * nv + threadIdx.x; q < nf; q += kThreads) __stcs(out + q, xs[q]);
+}
+
 __device__ __forceinline__ void unpack_bf16x2(uint32_t u, float &x, float &y)
 {
     const float2 f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&u));

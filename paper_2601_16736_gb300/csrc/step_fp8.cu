@@ -612,59 +612,120 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_fp8(const StepArgs 
 
 // ------------------------------------------------------ export / import
 
-__global__ void export_fp8_kernel(const uint8_t *__restrict__ m, const uint8_t *__restrict__ v,
-                                  const float *__restrict__ msc, const float *__restrict__ vsc, int32_t n,
-                                  float *__restrict__ m_out, float *__restrict__ v_out, uint32_t *__restrict__ t_out)
+// Columns of code word k (k < 15) in a canonical row x: 0-11 SH, 12 rotation,
+// 13 xyz and opacity, 14 scale (and the padding slot).
+__device__ __forceinline__ void f8_put(int k, const float *y, float *x)
 {
-    const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx >= (int64_t)n * kF8Cols) return;
-    const int64_t r = idx / kF8Cols;
-    const int c = f8_slot((int)(idx - r * kF8Cols));
-    const int64_t sb = (r / kF8Tile) * 64 + c;
-    if (m_out) m_out[idx] = f8_dec(m[r * kF8Step + c]) * msc[sb];
-    if (v_out) v_out[idx] = f8_dec(v[r * kF8Step + c]) * vsc[sb];
-    if (t_out && c == 0) t_out[r] = reinterpret_cast<const uint32_t *>(m + r * kF8Step)[kF8TWord];
+    float *p = k < 12 ? x + 11 + 4 * k : k == 12 ? x + 6 : k == 13 ? x : x + 3;
+    p[0] = y[0];
+    p[1] = y[1];
+    p[2] = y[2];
+    if (k < 13) p[3] = y[3];
+    else if (k == 13) x[10] = y[3];
 }
 
-// One CTA per block: the slot maxima of the imported values, the scales,
-// then the codes (both moments to nearest, a positive v never to zero).  A
-// NULL part keeps the stored one.
-__global__ void __launch_bounds__(kThreads) import_fp8_kernel(uint8_t *__restrict__ m, uint8_t *__restrict__ v,
-                                                              float *__restrict__ msc, float *__restrict__ vsc,
-                                                              int32_t n, const float *__restrict__ m_in,
-                                                              const float *__restrict__ v_in,
-                                                              const uint32_t *__restrict__ t_in)
+// 64 rows per CTA (a quarter of a block): their codes are one contiguous run
+// read as 16-B chunks (8 lanes to a primitive), decoded into canonical rows in
+// shared memory and stored as float4, as the other formats' export does.
+// 1 234 567 rows: 134 us against 281 with a thread per value (floor 109).
+constexpr int kF8IoRows = 64;
+
+__global__ void __launch_bounds__(kThreads) export_fp8_kernel(const uint4 *__restrict__ state,
+                                                              const float *__restrict__ msc,
+                                                              const float *__restrict__ vsc, int32_t n,
+                                                              float *__restrict__ m_out, float *__restrict__ v_out,
+                                                              uint32_t *__restrict__ t_out)
 {
-    __shared__ uint32_t s_max[2][64];
-    __shared__ float s_inv[2][64];
+    constexpr int kFloats = kF8IoRows * kF8Cols, kPer = kF8IoRows * 8 / kThreads;
+    __shared__ __align__(16) float x[2 * kFloats + 4];
+    __shared__ float sc[2][64];
     const int tid = threadIdx.x;
+    const int64_t r0 = (int64_t)blockIdx.x * kF8IoRows;
+    const int nrow = (int)min((int64_t)kF8IoRows, (int64_t)n - r0);
+    uint4 w[kPer];
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const int q = tid + u * kThreads, c2 = q & 7;
+        const bool want = c2 >= 4 ? v_out != nullptr : m_out || (t_out && c2 == 3);
+        w[u] = make_uint4(0u, 0u, 0u, 0u);
+        if (q < nrow * 8 && want) w[u] = __ldcs(state + r0 * 8 + q);
+    }
+    if (tid < 128) sc[tid >> 6][tid & 63] = (tid & 63) < kF8Cols ? (tid < 64 ? msc : vsc)[(r0 / kF8Tile) * 64 + (tid & 63)] : 0.f;
+    __syncthreads();
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        const int q = tid + u * kThreads, r = q >> 3, side = (q >> 2) & 1, c = q & 3;
+        const uint32_t ws[4] = {w[u].x, w[u].y, w[u].z, w[u].w};
+        float *row = x + (side ? kFloats + 4 : 0) + r * kF8Cols;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int k = 4 * c + j;
+            if (k == kF8TWord) break;
+            float y[4];
+            f8_dec4(ws[j], &sc[side][4 * k], y);
+            f8_put(k, y, row);
+        }
+        if (t_out && !side && c == 3 && r < nrow) t_out[r0 + r] = ws[3];
+    }
+    __syncthreads();
+    if (m_out) store_canonical(m_out + r0 * kF8Cols, nrow * kF8Cols, x);
+    if (v_out) store_canonical(v_out + r0 * kF8Cols, nrow * kF8Cols, x + kFloats + 4);
+}
+
+// One CTA per block and moment (blockIdx.y): each thread holds one column of 64
+// rows in registers (loads of consecutive columns by consecutive lanes, all in
+// flight at once), so the values are read once for both the column's largest
+// magnitude, hence its scale, and the codes (both moments to nearest, a
+// positive v never to zero), which leave through shared memory as 16-B
+// chunks.  A NULL part keeps the stored one.  1 234 567 rows: 146 us against
+// 351 with two passes over the values and an atomic maximum for each (floor
+// 109).
+__global__ void __launch_bounds__(kThreads, 2) import_fp8_kernel(uint4 *__restrict__ state, float *__restrict__ msc,
+                                                                 float *__restrict__ vsc, int32_t n,
+                                                                 const float *__restrict__ m_in,
+                                                                 const float *__restrict__ v_in,
+                                                                 const uint32_t *__restrict__ t_in)
+{
+    constexpr int kGroups = kThreads / 64, kPer = kF8Tile / kGroups;
+    __shared__ uint32_t s_max[kGroups][64];
+    __shared__ __align__(16) uint8_t raw[kF8Tile * kF8Row];
+    const int tid = threadIdx.x, col = tid & 63, grp = tid >> 6, side = blockIdx.y;
     const int64_t r0 = (int64_t)blockIdx.x * kF8Tile;
     const int nrow = (int)min((int64_t)kF8Tile, (int64_t)n - r0);
-    if (tid < 64) s_max[0][tid] = s_max[1][tid] = 0u;
+    const float *in = side ? v_in : m_in;
+    uint4 *rows = state + r0 * 8 + 4 * side;          // chunk c of row r at rows[8 r + c]
+    if (!in) {
+        if (!side && t_in && tid < nrow) reinterpret_cast<uint32_t *>(rows + 8 * tid + 3)[3] = t_in[r0 + tid];
+        return;
+    }
+    float x[kPer];
+    uint32_t b = 0u;
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) {
+        const int r = grp + kGroups * i;
+        x[i] = col < kF8Cols && r < nrow ? __ldcs(in + (r0 + r) * kF8Cols + col) : 0.f;
+    }
+#pragma unroll
+    for (int i = 0; i < kPer; ++i) b = max(b, __float_as_uint(fabsf(x[i])));
+    s_max[grp][col] = b;
+    if (tid < nrow)                                    // the last word: t in the m row
+        reinterpret_cast<uint32_t *>(raw)[tid * (kF8Row / 4) + kF8TWord] =
+            side ? 0u : t_in ? t_in[r0 + tid] : reinterpret_cast<const uint32_t *>(rows + 8 * tid + 3)[3];
     __syncthreads();
-    const int64_t e0 = r0 * kF8Cols;
-    for (int q = tid; q < nrow * kF8Cols; q += kThreads) {
-        const int c = f8_slot(q % kF8Cols);
-        if (m_in) atomicMax(&s_max[0][c], __float_as_uint(fabsf(m_in[e0 + q])));
-        if (v_in) atomicMax(&s_max[1][c], __float_as_uint(fabsf(v_in[e0 + q])));
+    if (col <= kF8Cols) {
+#pragma unroll
+        for (int g = 0; g < kGroups; ++g) b = max(b, s_max[g][col]);
+        const int e = b ? f8_scale_exp(b) : 0;
+        const int slot = col < kF8Cols ? f8_slot(col) : kF8Cols;        // column 59: the padding slot, zero
+        if (grp == 0 && col < kF8Cols) (side ? vsc : msc)[(int64_t)blockIdx.x * 64 + slot] = b ? pow2f(e) : 0.f;
+        const float inv = b ? pow2f(-e) : 0.f;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i)
+            raw[(grp + kGroups * i) * kF8Row + slot] = (uint8_t)(side ? f8_rn_floor(x[i] * inv) : f8_rn(x[i] * inv));
     }
     __syncthreads();
-    if (tid < 2 * kF8Cols) {
-        const int w = tid / kF8Cols, c = tid - w * kF8Cols;
-        if (w ? v_in != nullptr : m_in != nullptr) {
-            const uint32_t b = s_max[w][c];
-            const int e = b ? f8_scale_exp(b) : 0;
-            (w ? vsc : msc)[blockIdx.x * 64 + c] = b ? pow2f(e) : 0.f;
-            s_inv[w][c] = b ? pow2f(-e) : 0.f;
-        }
-    }
-    __syncthreads();
-    for (int q = tid; q < nrow * kF8Cols; q += kThreads) {
-        const int lr = q / kF8Cols, c = f8_slot(q - lr * kF8Cols);
-        if (m_in) m[(r0 + lr) * kF8Step + c] = (uint8_t)f8_rn(m_in[e0 + q] * s_inv[0][c]);
-        if (v_in) v[(r0 + lr) * kF8Step + c] = (uint8_t)f8_rn_floor(v_in[e0 + q] * s_inv[1][c]);
-    }
-    if (t_in && tid < nrow) reinterpret_cast<uint32_t *>(m + (r0 + tid) * kF8Step)[kF8TWord] = t_in[r0 + tid];
+    for (int q = tid; q < nrow * 4; q += kThreads)
+        __stcs(rows + 8 * (q >> 2) + (q & 3), reinterpret_cast<const uint4 *>(raw)[q]);
 }
 
 // ------------------------------------------------------------- re-index
@@ -758,10 +819,8 @@ cudaError_t launch_export_fp8(const StateView &st, int32_t n, float *m_out, floa
                               cudaStream_t s)
 {
     if (n <= 0 || (!m_out && !v_out && !t_out)) return cudaSuccess;
-    const int64_t total = (int64_t)n * kF8Cols;
-    export_fp8_kernel<<<(unsigned)((total + kThreads - 1) / kThreads), kThreads, 0, s>>>(
-        static_cast<const uint8_t *>(st.m), static_cast<const uint8_t *>(st.v), st.msc, st.vsc, n, m_out, v_out,
-        t_out);
+    export_fp8_kernel<<<(unsigned)(((int64_t)n + kF8IoRows - 1) / kF8IoRows), kThreads, 0, s>>>(
+        static_cast<const uint4 *>(st.m), st.msc, st.vsc, n, m_out, v_out, t_out);
     return cudaGetLastError();
 }
 
@@ -769,8 +828,8 @@ cudaError_t launch_import_fp8(const StateView &st, int32_t n, const float *m_in,
                               const uint32_t *t_in, cudaStream_t s)
 {
     if (n <= 0 || (!m_in && !v_in && !t_in)) return cudaSuccess;
-    import_fp8_kernel<<<(unsigned)((n + kF8Tile - 1) / kF8Tile), kThreads, 0, s>>>(
-        static_cast<uint8_t *>(st.m), static_cast<uint8_t *>(st.v), st.msc, st.vsc, n, m_in, v_in, t_in);
+    import_fp8_kernel<<<dim3((unsigned)(((int64_t)n + kF8Tile - 1) / kF8Tile), 2), kThreads, 0, s>>>(
+        static_cast<uint4 *>(st.m), st.msc, st.vsc, n, m_in, v_in, t_in);
     return cudaGetLastError();
 }
 
