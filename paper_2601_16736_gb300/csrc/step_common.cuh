@@ -577,21 +577,39 @@ __device__ __forceinline__ void prefetch_row_l2(const StepArgs &a, int32_t row)
                  "n"(2 * kRowBytes) : "memory");
 }
 
+// Tiles of a launch.  CTA b takes `rows` rows from `first`: kTile rows for the
+// first a.n_big CTAs, then a.tail_rows (a multiple of 16) each.
+struct TileSpan {
+    int64_t first;
+    int rows;
+};
+template <int kTile>
+__device__ __forceinline__ TileSpan tile_span(const StepArgs &a, const int64_t b)
+{
+    const int64_t t = b - a.n_big;
+    if (t < 0) return {b * kTile, kTile};
+    const int64_t first = (int64_t)a.n_big * kTile + t * a.tail_rows;
+    return {first, (int)min((int64_t)a.tail_rows, (int64_t)a.n_rows - first)};
+}
+
 // Ask L2 for the visibility inputs (means or mask bytes) of the tile one wave
 // of resident CTAs ahead: the tile that starts when a slot frees, whose
 // phase A then finds them on chip instead of waiting a DRAM round trip.  A
-// hint only; nothing waits for it.  Whole tiles only, 16-B aligned sources.
+// hint only; nothing waits for it.  16-B multiples from 16-B aligned sources
+// (tiles start on a multiple of 16 rows; the last one may be ragged).
 template <int kTile>
 __device__ __forceinline__ void prefetch_tile_ahead(const StepArgs &a, const int vis_src)
 {
-    static_assert((kTile * 12) % 16 == 0 && kTile % 16 == 0, "bulk prefetch sizes are multiples of 16 B");
+    static_assert(kTile % 16 == 0, "bulk prefetch sizes are multiples of 16 B");
     if (threadIdx.x != 0 || a.tile_ahead <= 0) return;
-    const int64_t q = ((int64_t)blockIdx.x + a.tile_ahead) * kTile;
-    if (q + kTile > (int64_t)a.n_rows) return;
+    const TileSpan t = tile_span<kTile>(a, (int64_t)blockIdx.x + a.tile_ahead);
+    if (t.rows < 16) return;
+    const uint32_t rows = (uint32_t)t.rows & ~15u;
     if (vis_src == kVisCamera && ((uintptr_t)a.a_xyz & 15u) == 0)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.a_xyz + q * 3), "n"(kTile * 12) : "memory");
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.a_xyz + t.first * 3), "r"(rows * 12)
+                     : "memory");
     else if (vis_src == kVisMask && ((uintptr_t)a.mask_in & 15u) == 0)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.mask_in + q), "n"(kTile) : "memory");
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.mask_in + t.first), "r"(rows) : "memory");
 }
 
 // CTAs of kernel `fn` (kThreads threads, static shared memory only) resident
@@ -614,29 +632,62 @@ inline int resident_ctas(const void *fn, int *cache)
     return c;
 }
 
-// Prefetch when at most 60 % of the tile's rows are visible.
 // Beside the means: ask L2 for what phase A of the tile one wave ahead reads
 // for its rows, so that its loads find them on chip: the opacity logits when
 // counting N_a or drawing noise, and the rotations and log-scales for noise.
-// A hint only; whole tiles, 16-B aligned sources.
+// A hint only; 16-B multiples from 16-B aligned sources.
 template <int kTile>
 __device__ __forceinline__ void prefetch_tile_ahead_x(const StepArgs &a)
 {
     if (threadIdx.x != 0 || a.tile_ahead <= 0 || !(a.n_active || a.noise)) return;
-    const int64_t q = ((int64_t)blockIdx.x + a.tile_ahead) * kTile;
-    if (q + kTile > (int64_t)a.n_rows) return;
+    const TileSpan t = tile_span<kTile>(a, (int64_t)blockIdx.x + a.tile_ahead);
+    if (t.rows < 16) return;
+    const int64_t q = t.first;
+    const uint32_t rows = (uint32_t)t.rows & ~15u;
     if (((uintptr_t)a.a_op & 15u) == 0)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.a_op + q), "n"(kTile * 4) : "memory");
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.a_op + q), "r"(rows * 4) : "memory");
     if (a.noise) {
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.a_rot + q * 4), "n"(kTile * 16) : "memory");
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.a_rot + q * 4), "r"(rows * 16) : "memory");
         if (((uintptr_t)a.a_scale & 15u) == 0)
-            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.a_scale + q * 3), "n"(kTile * 12)
+            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.a_scale + q * 3), "r"(rows * 12)
                          : "memory");
     }
 }
 
+// Prefetch when at most 60 % of the tile's rows are visible.
+__device__ __forceinline__ bool sparse_tile(int nv, int rows) { return 5 * nv <= 3 * rows; }
+
+// The grid of a step over a.n_rows rows in CTAs of up to kTile rows, `resident`
+// of them at once, and its tile sizes (a.n_big, a.tail_rows).  A tile of 256
+// rows is the best size for a large sparse scene (128: 1.1-1.3 times the time
+// at 10-20 % visible, where a tile's items no longer fill its threads).  But a
+// scene that makes fewer tiles than the chip holds leaves it idle, and a large
+// one ends in a wave that is partly empty:
+//   * up to one wave of 256-row tiles, 128 rows to a CTA, and up to one wave
+//     of 64-row tiles, 64 rows (FP32, 88 % visible: 20 k rows 9.6 us against
+//     14.8, 100 k 28.9 against 33.1; 30 % visible: 9.3 against 9.8, 13.5
+//     against 16.9);
+//   * beyond, the rows of the last half wave in 128-row tiles (1 M rows, 30 %
+//     visible: FP32 108.9 us against 109.9, BF16 at 777 k 66.6 against 68.0;
+//     88 % visible: FP32 279.7 against 285.7; 3 M and 6 M rows level).
 template <int kTile>
-__device__ __forceinline__ bool sparse_tile(int nv) { return 5 * nv <= 3 * kTile; }
+inline unsigned plan_tiles(StepArgs &a, const int resident)
+{
+    const int64_t n = a.n_rows, wave = resident;
+    a.tile_ahead = resident;
+    a.tail_rows = n <= wave * (kTile / 4) ? kTile / 4 : kTile / 2;
+    a.n_big = n <= wave * kTile ? 0 : (int32_t)(n / kTile - wave / 2);
+    return (unsigned)(a.n_big + (n - (int64_t)a.n_big * kTile + a.tail_rows - 1) / a.tail_rows);
+}
+
+// FP32: the visible rows of a tile whose items run together (768 SH items, then
+// their small items) before the next rows'.  A row's last moment line holds both
+// SH and small columns, so the two should follow each other while the line is
+// in L2; with the tiles in flight of a dense scene larger than L2, it came and
+// went twice (1 M rows, 88 % visible: 269 us against 285; 30 %: level).  The
+// 16-bit formats take the whole tile as one group: the loop over groups costs
+// them registers (BF16, 30 % visible: 78 us against 68).
+constexpr int kGroupRows = 64;
 
 // Small items per row: rotation; xyz + scale0; scale1 + scale2 + opacity,
 // except FP16-block rows (rotation; xyz + scale + opacity).

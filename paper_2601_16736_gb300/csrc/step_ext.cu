@@ -6,7 +6,7 @@
 // the terms form of the plain step kernel, and the plain step is untouched
 // by any of them.
 //
-// Per tile of 256 rows (one CTA of 256 threads; 5 CTAs per SM for FP32 and
+// Per tile of up to 256 rows (one CTA of 256 threads; 5 CTAs per SM for FP32 and
 // BF16 moments, 4 for the others):
 //   A. visibility, StSS, AIU and noise decisions per row.  A row that takes
 //      the noise has it computed here, from its values before this step, and
@@ -297,13 +297,14 @@ __device__ __forceinline__ float2 factors(const StepArgs &a, uint32_t k)
 
 // Phase A of the extended step; returns the two list lengths.
 template <int kTile, int kRowBytes, int kTByte>
-__device__ __forceinline__ void tile_decide_x(const StepArgs &a, const int vis_src, const int64_t r0,
+__device__ __forceinline__ void tile_decide_x(const StepArgs &a, const int vis_src, const TileSpan span,
                                               TileListsX<kTile> &L, int &nv, int &ni)
 {
     constexpr int kRpt = kTile / kThreads;
     constexpr int kWarps = kThreads / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nrow = (int)min((int64_t)kTile, (int64_t)a.n_rows - r0);
+    const int64_t r0 = span.first;
+    const int nrow = span.rows;
     unsigned bal_v[kRpt], bal_i[kRpt];
     uint8_t flag[kRpt];
     uint32_t t_old[kRpt];
@@ -382,7 +383,7 @@ __device__ __forceinline__ void tile_decide_x(const StepArgs &a, const int vis_s
         if (bal_v[j] & me_bit) {
             const int pos = bv + __popc(bal_v[j] & lt);
             L.list[pos] = row;
-            if (sparse_tile<kTile>(nv)) prefetch_row_l2<kRowBytes>(a, row);
+            if (sparse_tile(nv, nrow)) prefetch_row_l2<kRowBytes>(a, row);
             L.vflag[pos] = flag[j];
             L.fac[pos] = factors(a, a.bias_mode ? a.k_bias : t_old[j] + 1u);
             L.nz[pos] = nz[j];
@@ -410,29 +411,39 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_x(const StepAr
     pdl_enter();
     prefetch_tile_ahead<kTile>(a, vis_src);
     prefetch_tile_ahead_x<kTile>(a);
-    const int64_t r0 = (int64_t)blockIdx.x * kTile;
     int nv, ni;
-    tile_decide_x<kTile, S::kRowBytes, S::kTByte>(a, vis_src, r0, L, nv, ni);
+    tile_decide_x<kTile, S::kRowBytes, S::kTByte>(a, vis_src, tile_span<kTile>(a, blockIdx.x), L, nv, ni);
 
     unsigned my_active = 0;
     constexpr int kSmall = kSmallItems<kPrec>, kOpItem = 11 + kSmall;     // the item holding the opacity
-    const int e_sh = kNsh * nv, e_vis = e_sh + kSmall * nv, e_ish = e_vis + kNsh * ni, e_all = e_ish + kSmall * ni;
+    const int e0 = kPrec == GS_MOM_FP32 ? 0 : (kNsh + kSmall) * nv;
+    const int e_ish = e0 + kNsh * ni, e_all = e_ish + kSmall * ni;
     // One flat item space walked as four loops, one per item kind, with the
     // item-to-thread assignment a single loop would give: the kinds do not
     // share a loop body, so their register demands do not add up.
     int w = threadIdx.x;
-    for (; w < e_sh; w += kThreads) {
-        const int j = w / kNsh, i = w - j * kNsh;
-        sh_item<kPrec, kW>(a, L.list[j], i, (L.vflag[j] & kFRsr) != 0, L.fac[j]);
-    }
-    for (; w < e_vis; w += kThreads) {
-        const int q = w - e_sh;
-        const int j = q % nv, c = 12 + q / nv;
-        const bool act = small_item_x<kPrec>(a, L.list[j], c, true, L.vflag[j], L.fac[j], L.nz[j]);
-        my_active += (c == kOpItem && act) ? 1u : 0u;
+    // the items of visible rows j0 .. j0+ng-1 of the list
+    auto run = [&](const int j0, const int ng) {
+        const int e_sh = kNsh * ng, e_vis = (kNsh + kSmall) * ng;
+        for (; w < e_sh; w += kThreads) {
+            const int q = w / kNsh, i = w - q * kNsh, j = j0 + q;
+            sh_item<kPrec, kW>(a, L.list[j], i, (L.vflag[j] & kFRsr) != 0, L.fac[j]);
+        }
+        for (; w < e_vis; w += kThreads) {
+            const int q = w - e_sh;
+            const int j = j0 + q % ng, c = 12 + q / ng;
+            const bool act = small_item_x<kPrec>(a, L.list[j], c, true, L.vflag[j], L.fac[j], L.nz[j]);
+            my_active += (c == kOpItem && act) ? 1u : 0u;
+        }
+        if constexpr (kPrec == GS_MOM_FP32) w -= e_vis;
+    };
+    if constexpr (kPrec == GS_MOM_FP32) {
+        for (int j0 = 0; j0 < nv; j0 += kGroupRows) run(j0, min(nv - j0, kGroupRows));
+    } else {
+        run(0, nv);
     }
     for (; w < e_ish; w += kThreads) {
-        const int q = w - e_vis;
+        const int q = w - e0;
         const int j = q / kNsh, i = q - j * kNsh;
         inv_sh_item<kPrec, kW>(a, L.ilist[j], i, L.iflag[j], L.ifac[j]);
     }
@@ -467,8 +478,7 @@ cudaError_t launch_ext_t(const StepArgs &a, int vis_src, cudaStream_t s)
     auto k = step_tile_x<kExtTile, kExtMinBlocks<kPrec>, kPrec, kW>;
     static int s_res[64] = {};
     StepArgs b = a;
-    b.tile_ahead = resident_ctas(reinterpret_cast<const void *>(k), s_res);
-    const unsigned grid = (unsigned)((a.n_rows + kExtTile - 1) / kExtTile);
+    const unsigned grid = plan_tiles<kExtTile>(b, resident_ctas(reinterpret_cast<const void *>(k), s_res));
     return launch_pdl(k, grid, kThreads, s, b, vis_src);
 }
 

@@ -2,7 +2,8 @@
 // visible rows of a tile, Sparse Adam + DAR on the visible rows, RSR on the
 // StSS-sampled rows — one pass over HBM per step.
 //
-// One CTA handles one tile of kTile consecutive rows with 256 threads:
+// One CTA handles one tile of up to kTile consecutive rows (plan_tiles) with 256
+// threads:
 //   A. each thread decides visibility (camera frustum test of the mean,
 //      caller mask, or all-visible) and StSS membership for kTile/256 rows,
 //      issuing the load of a visible row's step counter right away; warp
@@ -58,13 +59,14 @@ struct TileTerms {
 // go to X beside its list entry, and invisible rows, whose opacity this step
 // leaves unchanged, are counted into X->active when the step counts N_a.
 template <int kTile, int kRowBytes, int kTByte, bool kX>
-__device__ __forceinline__ void tile_decide(const StepArgs &a, const int vis_src, const int64_t r0, TileLists<kTile> &L,
-                                            TileTerms<kTile> *X, int &nv, int &nr)
+__device__ __forceinline__ void tile_decide(const StepArgs &a, const int vis_src, const TileSpan span,
+                                            TileLists<kTile> &L, TileTerms<kTile> *X, int &nv, int &nr)
 {
     constexpr int kRpt = kTile / kThreads;
     constexpr int kWarps = kThreads / 32;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nrow = (int)min((int64_t)kTile, (int64_t)a.n_rows - r0);
+    const int64_t r0 = span.first;
+    const int nrow = span.rows;
     unsigned bal_v[kRpt], bal_r[kRpt], bal_s[kRpt];
     uint32_t t_old[kRpt];
     float4 xq[kX ? kRpt : 1], xs[kX ? kRpt : 1];
@@ -140,7 +142,7 @@ __device__ __forceinline__ void tile_decide(const StepArgs &a, const int vis_src
             const bool smp = (bal_s[j] >> lane) & 1u;
             const int pos = bv + __popc(bal_v[j] & lt);
             L.list[pos] = row | (smp ? (int32_t)0x80000000 : 0);
-            if (sparse_tile<kTile>(nv)) prefetch_row_l2<kRowBytes>(a, row);
+            if (sparse_tile(nv, nrow)) prefetch_row_l2<kRowBytes>(a, row);
             const uint32_t tb = a.bias_mode ? a.k_bias : t_old[j] + 1u;
             L.fac[pos] = (tb < (uint32_t)a.fac_len) ? a.fac[tb] : make_float2(1.0f, 1.0f);
             if constexpr (kX) { if (a.noise) { X->q[pos] = xq[j]; X->sko[pos] = xs[j]; } }
@@ -154,44 +156,54 @@ __device__ __forceinline__ void tile_decide(const StepArgs &a, const int vis_src
 // ---------------------------------------------------------------- the kernel
 
 // Phase B of one tile: the items of its visible and invisible-sampled rows
-// (nv, nr of them in L), grouped by kind: all SH items, then the small
-// items, then RSR.  kX: the xyz items draw the rows' noise from the values
-// kept in X and subtract it, the opacity items count the rows active after
-// the step, and the tile's count is added to a.n_active.
+// (nv, nr of them in L), grouped by kind: SH items, then small items (FP32:
+// group of rows by group of rows), then RSR.  kX: the xyz items draw the rows' noise
+// from the values kept in X and subtract it, the opacity items count the rows
+// active after the step, and the tile's count is added to a.n_active.
 template <int kTile, int kPrec, int kW, bool kX>
 __device__ __forceinline__ void tile_items(const StepArgs &a, const TileLists<kTile> &L, TileTerms<kTile> *X,
                                            const int nv, const int nr)
 {
     constexpr int kNsh = 48 / kW, kItems = kNsh + kSmallItems<kPrec>;
-    const int e_sh = kNsh * nv, e_vis = kItems * nv, e_all = e_vis + kItems * nr;
     // One flat item space, walked as three loops (SH items, small items, RSR
     // items) with the same item-to-thread assignment as a single loop: the
-    // kinds no longer share a loop body, so their register demands do not
-    // add up (FP16 block then fits 5 CTAs per SM).
+    // kinds do not share a loop body, so their register demands do not add up
+    // (FP16 block then fits 5 CTAs per SM).
     unsigned my_active = 0;
     int w = threadIdx.x;
-    for (; w < e_sh; w += kThreads) {
-        const int j = w / kNsh, i = w - j * kNsh;
-        const int32_t e = L.list[j];
-        sh_item<kPrec, kW>(a, e & 0x7fffffff, i, e < 0, L.fac[j]);
-    }
-    for (; w < e_vis; w += kThreads) {
-        const int q = w - e_sh;
-        const int j = q % nv, c = 12 + q / nv;
-        const int32_t e = L.list[j];
-        if constexpr (kX) {
-            float3 nz = make_float3(0.f, 0.f, 0.f);
-            if (c == 13 && a.noise) {
-                const float4 q = X->q[j], s4 = X->sko[j];
-                nz = noise_term(a, e & 0x7fffffff, q, s4.x, s4.y, s4.z, s4.w);
-            }
-            my_active += small_item<kPrec, true>(a, e & 0x7fffffff, c, e < 0, L.fac[j], nz) ? 1u : 0u;
-        } else {
-            small_item<kPrec>(a, e & 0x7fffffff, c, e < 0, L.fac[j]);
+    // the items of rows j0 .. j0+ng-1 of the list
+    auto run = [&](const int j0, const int ng) {
+        const int e_sh = kNsh * ng, e_vis = kItems * ng;
+        for (; w < e_sh; w += kThreads) {
+            const int q = w / kNsh, i = w - q * kNsh, j = j0 + q;
+            const int32_t e = L.list[j];
+            sh_item<kPrec, kW>(a, e & 0x7fffffff, i, e < 0, L.fac[j]);
         }
+        for (; w < e_vis; w += kThreads) {
+            const int q = w - e_sh;
+            const int j = j0 + q % ng, c = 12 + q / ng;
+            const int32_t e = L.list[j];
+            if constexpr (kX) {
+                float3 nz = make_float3(0.f, 0.f, 0.f);
+                if (c == 13 && a.noise) {
+                    const float4 q4 = X->q[j], s4 = X->sko[j];
+                    nz = noise_term(a, e & 0x7fffffff, q4, s4.x, s4.y, s4.z, s4.w);
+                }
+                my_active += small_item<kPrec, true>(a, e & 0x7fffffff, c, e < 0, L.fac[j], nz) ? 1u : 0u;
+            } else {
+                small_item<kPrec>(a, e & 0x7fffffff, c, e < 0, L.fac[j]);
+            }
+        }
+        if constexpr (kPrec == GS_MOM_FP32) w -= e_vis;
+    };
+    if constexpr (kPrec == GS_MOM_FP32) {
+        for (int j0 = 0; j0 < nv; j0 += kGroupRows) run(j0, min(nv - j0, kGroupRows));
+    } else {
+        run(0, nv);
     }
+    const int e0 = kPrec == GS_MOM_FP32 ? 0 : kItems * nv, e_all = e0 + kItems * nr;
     for (; w < e_all; w += kThreads) {
-        const int q = w - e_vis;
+        const int q = w - e0;
         const int j = q / kItems, i = q - j * kItems;
         rsr_item<kPrec, kW>(a, L.rlist[j], i);
     }
@@ -207,14 +219,14 @@ __device__ __forceinline__ void tile_items(const StepArgs &a, const TileLists<kT
 
 // One tile: phase A, then its items.
 template <int kTile, int kPrec, int kW, bool kX = false>
-__device__ __forceinline__ void process_tile(const StepArgs &a, const int vis_src, const int64_t r0,
+__device__ __forceinline__ void process_tile(const StepArgs &a, const int vis_src, const TileSpan span,
                                              TileLists<kTile> &L, TileTerms<kTile> *X = nullptr)
 {
     static_assert(kTile % kThreads == 0, "tile must be a multiple of the block");
     static_assert(kW == 4 || kW == 8, "SH items cover 4 or 8 columns");
     using S = State<kPrec>;
     int nv, nr;
-    tile_decide<kTile, S::kRowBytes, S::kTByte, kX>(a, vis_src, r0, L, X, nv, nr);
+    tile_decide<kTile, S::kRowBytes, S::kTByte, kX>(a, vis_src, span, L, X, nv, nr);
     tile_items<kTile, kPrec, kW, kX>(a, L, X, nv, nr);
 }
 
@@ -224,7 +236,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile(const StepArgs
     __shared__ TileLists<kTile> L;
     pdl_enter();
     prefetch_tile_ahead<kTile>(a, vis_src);
-    process_tile<kTile, kPrec, kW>(a, vis_src, (int64_t)blockIdx.x * kTile, L);
+    process_tile<kTile, kPrec, kW>(a, vis_src, tile_span<kTile>(a, blockIdx.x), L);
 }
 
 // The terms form: the same step with the active count N_a (Sec. 4) and/or
@@ -238,7 +250,15 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_terms(const St
     pdl_enter();
     prefetch_tile_ahead<kTile>(a, vis_src);
     prefetch_tile_ahead_x<kTile>(a);
-    process_tile<kTile, kPrec, kW, true>(a, vis_src, (int64_t)blockIdx.x * kTile, L, &X);
+    process_tile<kTile, kPrec, kW, true>(a, vis_src, tile_span<kTile>(a, blockIdx.x), L, &X);
+}
+
+// Tile t of a scene of a batch: kTile rows, the last one what is left.
+template <int kTile>
+__device__ __forceinline__ TileSpan whole_tile(const StepArgs &a, const int t)
+{
+    const int64_t first = (int64_t)t * kTile;
+    return {first, (int)min((int64_t)kTile, (int64_t)a.n_rows - first)};
 }
 
 // Many scenes in one persistent launch.  The scene table lives in device
@@ -276,7 +296,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_batch(const BatchPa
             cur = lo;
             __syncthreads();
         }
-        process_tile<kTile, kPrec, kW>(sa, kVisCamera, (int64_t)(t - p->tile_start[lo]) * kTile, L);
+        process_tile<kTile, kPrec, kW>(sa, kVisCamera, whole_tile<kTile>(sa, t - p->tile_start[lo]), L);
         __syncthreads();                       // the lists are reused by the next tile
     }
     if (tid == 0 && atomicAdd(done, 1u) == gridDim.x - 1) {
@@ -307,7 +327,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_batch_grid(const Ba
     uint32_t *dst = reinterpret_cast<uint32_t *>(&sa);
     for (int q = threadIdx.x; q < (int)(sizeof(StepArgs) / 4); q += kThreads) dst[q] = src[q];
     __syncthreads();
-    process_tile<kTile, kPrec, kW>(sa, kVisCamera, (int64_t)(t - p->tile_start[lo]) * kTile, L);
+    process_tile<kTile, kPrec, kW>(sa, kVisCamera, whole_tile<kTile>(sa, t - p->tile_start[lo]), L);
 }
 
 }  // namespace
@@ -335,9 +355,8 @@ cudaError_t launch_tiles(const StepArgs &a, int vis_src, cudaStream_t s)
                 : step_tile<kStepTile, kStepMinBlocks<kPrec>, kPrec, kW>;
     static int s_res[64] = {};
     StepArgs b = a;
-    b.tile_ahead = resident_ctas(reinterpret_cast<const void *>(k), s_res);
-    const unsigned n_tiles = (unsigned)((a.n_rows + kStepTile - 1) / kStepTile);
-    return launch_pdl(k, n_tiles, kThreads, s, b, vis_src);
+    const unsigned grid = plan_tiles<kStepTile>(b, resident_ctas(reinterpret_cast<const void *>(k), s_res));
+    return launch_pdl(k, grid, kThreads, s, b, vis_src);
 }
 
 }  // namespace
