@@ -1,7 +1,8 @@
 """The step's tile sizes change with the number of rows (64, 128 or 256 rows to
-a CTA, and smaller tiles at the end of a large grid).  The tiling must not show
-in the results: bit for bit those of the batched step, which cuts a scene into
-whole tiles, at sizes on both sides of every edge."""
+a CTA, and smaller tiles at the end of a large grid; FP8: 256 or 512 threads to
+a block).  The tiling must not show in the results: bit for bit those of the
+batched step, which cuts a scene into whole tiles, at sizes on both sides of
+every edge."""
 import numpy as np
 import pytest
 
@@ -64,3 +65,25 @@ def test_tiling_does_not_change_the_step(G, prec, waves, tile, extra):
     batch.close()
     for r in (one, cut, terms):
         r.close()
+
+
+def test_fp8_block_width_does_not_change_the_step(G):
+    """The same blocks in a scene small enough for 512 threads a block and in
+    one with a block more, which takes 256."""
+    n = 2 * _sms() * 256
+    groups = synth.scene_blobs(n + 256, 79, 12.5)
+    grads = synth.grads_rows(n + 256, 80)
+    small = GpuScene({k: x[:n] for k, x in groups.items()}, prec=G.GS_MOM_FP8E4M3)
+    large = GpuScene(groups, prec=G.GS_MOM_FP8E4M3)
+    small.set_grads(grads[:n])
+    large.set_grads(grads)
+    cams = synth.ring_cameras(10, (0.0,))
+    for k in range(1, 5):
+        p = G.make_params(synth.lr_for_step(k, 10), k, restate=(k == 2), restate_ratio=0.3, seed=5)
+        small.step_camera(cams[k], p)
+        large.step_camera(cams[k], p)
+    assert large.rows()[:n].tobytes() == small.rows().tobytes()
+    for a, b in zip(small.state(), large.state()):
+        assert a.tobytes() == b[:n].tobytes()
+    small.close()
+    large.close()
