@@ -436,14 +436,10 @@ gs_status gs_visibility(gs_opt *o, const float *xyz, const gs_camera *cam, uint8
         !dev_ok(o, n_visible, n_visible ? 8 : 0, 8))
         return GS_ERR_INVALID_ARG;
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    cudaError_t e = cudaSuccess;
     float c[gs::kCamFloats];
     gs::camera_arg(reinterpret_cast<const float *>(cam), c);
-    if (n_visible) e = cudaMemsetAsync(n_visible, 0, 8, s);
-    if (e == cudaSuccess)
-        e = gs::launch_visibility(xyz, (int32_t)n, c, mask, visible_rows,
-                                  reinterpret_cast<unsigned long long *>(n_visible), s);
-    return fail_cuda(o, e);
+    return fail_cuda(o, gs::launch_visibility(xyz, (int32_t)n, c, mask, visible_rows,
+                                              reinterpret_cast<unsigned long long *>(n_visible), s));
 }
 
 gs_status gs_step(gs_opt *o, const gs_attrs *attrs, const gs_grads *grads, const uint8_t *mask,

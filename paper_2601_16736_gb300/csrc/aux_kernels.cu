@@ -58,6 +58,14 @@ __global__ void __launch_bounds__(kThreads) visibility_kernel(const float *__res
     }
 }
 
+// The count starts from zero.  A kernel in the launch chain rather than a memset:
+// the filter's CTAs are then already resident when the zero is written.
+__global__ void zero_count_kernel(unsigned long long *count)
+{
+    pdl_enter();
+    *count = 0ull;
+}
+
 // Eight consecutive rows per thread, for 16-B aligned means: six float4
 // loads carry the rows' 24 values, two 32-bit stores their mask bytes.  The
 // CTA's visible rows are placed by an exclusive scan of the per-thread
@@ -441,6 +449,10 @@ unsigned blocks_for(int64_t n_threads) { return (unsigned)((n_threads + kThreads
 cudaError_t launch_visibility(const float *xyz, int32_t n, const float cam[kCamFloats], uint8_t *mask, int32_t *list,
                               unsigned long long *count, cudaStream_t s)
 {
+    if (count) {
+        const cudaError_t e = launch_pdl(zero_count_kernel, 1u, 1u, s, count);
+        if (e != cudaSuccess) return e;
+    }
     if (n <= 0) return cudaSuccess;
     CamArg c;
     memcpy(c.c, cam, sizeof(c.c));
