@@ -92,7 +92,7 @@ struct StepArgs {
     unsigned long long *n_active;   // optional, accumulated with atomicAdd
     int32_t g_host;              // gradients are pinned host memory read in place
     int32_t tile_ahead;          // CTAs resident at once (0: no look-ahead prefetch)
-    int32_t n_big, tail_rows;    // tiles of the launch (tile_span)
+    int32_t n_big, big_rows, tail_rows;   // tiles of the launch (tile_span)
     float *msc, *vsc;            // FP8 moments: per-(256-row block, column) scales of m, v
 };
 

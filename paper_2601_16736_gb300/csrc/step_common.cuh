@@ -577,18 +577,17 @@ __device__ __forceinline__ void prefetch_row_l2(const StepArgs &a, int32_t row)
                  "n"(2 * kRowBytes) : "memory");
 }
 
-// Tiles of a launch.  CTA b takes `rows` rows from `first`: kTile rows for the
-// first a.n_big CTAs, then a.tail_rows (a multiple of 16) each.
+// Tiles of a launch.  CTA b takes `rows` rows from `first`: a.big_rows rows for
+// the first a.n_big CTAs, then a.tail_rows each (both multiples of 16).
 struct TileSpan {
     int64_t first;
     int rows;
 };
-template <int kTile>
 __device__ __forceinline__ TileSpan tile_span(const StepArgs &a, const int64_t b)
 {
     const int64_t t = b - a.n_big;
-    if (t < 0) return {b * kTile, kTile};
-    const int64_t first = (int64_t)a.n_big * kTile + t * a.tail_rows;
+    if (t < 0) return {b * a.big_rows, a.big_rows};
+    const int64_t first = (int64_t)a.n_big * a.big_rows + t * a.tail_rows;
     return {first, (int)min((int64_t)a.tail_rows, (int64_t)a.n_rows - first)};
 }
 
@@ -597,12 +596,10 @@ __device__ __forceinline__ TileSpan tile_span(const StepArgs &a, const int64_t b
 // phase A then finds them on chip instead of waiting a DRAM round trip.  A
 // hint only; nothing waits for it.  16-B multiples from 16-B aligned sources
 // (tiles start on a multiple of 16 rows; the last one may be ragged).
-template <int kTile>
 __device__ __forceinline__ void prefetch_tile_ahead(const StepArgs &a, const int vis_src)
 {
-    static_assert(kTile % 16 == 0, "bulk prefetch sizes are multiples of 16 B");
     if (threadIdx.x != 0 || a.tile_ahead <= 0) return;
-    const TileSpan t = tile_span<kTile>(a, (int64_t)blockIdx.x + a.tile_ahead);
+    const TileSpan t = tile_span(a, (int64_t)blockIdx.x + a.tile_ahead);
     if (t.rows < 16) return;
     const uint32_t rows = (uint32_t)t.rows & ~15u;
     if (vis_src == kVisCamera && ((uintptr_t)a.a_xyz & 15u) == 0)
@@ -636,11 +633,10 @@ inline int resident_ctas(const void *fn, int *cache)
 // for its rows, so that its loads find them on chip: the opacity logits when
 // counting N_a or drawing noise, and the rotations and log-scales for noise.
 // A hint only; 16-B multiples from 16-B aligned sources.
-template <int kTile>
 __device__ __forceinline__ void prefetch_tile_ahead_x(const StepArgs &a)
 {
     if (threadIdx.x != 0 || a.tile_ahead <= 0 || !(a.n_active || a.noise)) return;
-    const TileSpan t = tile_span<kTile>(a, (int64_t)blockIdx.x + a.tile_ahead);
+    const TileSpan t = tile_span(a, (int64_t)blockIdx.x + a.tile_ahead);
     if (t.rows < 16) return;
     const int64_t q = t.first;
     const uint32_t rows = (uint32_t)t.rows & ~15u;
@@ -665,8 +661,11 @@ __device__ __forceinline__ bool sparse_tile(int nv, int rows) { return 5 * nv <=
 // one ends in a wave that is partly empty:
 //   * up to one wave of 256-row tiles, 128 rows to a CTA, and up to one wave
 //     of 64-row tiles, 64 rows (FP32, 88 % visible: 20 k rows 9.6 us against
-//     14.8, 100 k 28.9 against 33.1; 30 % visible: 9.3 against 9.8, 13.5
-//     against 16.9);
+//     14.8, 190 k 52.6 against 60; 30 % visible: 20 k rows 9.3 against 9.8,
+//     190 k level);
+//   * of those, what makes 1 to 1.4 waves of 128 rows ends in a quarter of its
+//     rows by 64 (100 k rows, 88 % visible: 24.2 us against 27.8 for 128 rows
+//     throughout and 33.1 for 256; 30 % visible: level, and 16.9 for 256);
 //   * beyond, the rows of the last half wave in 128-row tiles (1 M rows, 30 %
 //     visible: FP32 108.9 us against 109.9, BF16 at 777 k 66.6 against 68.0;
 //     88 % visible: FP32 279.7 against 285.7; 3 M and 6 M rows level).
@@ -675,9 +674,19 @@ inline unsigned plan_tiles(StepArgs &a, const int resident)
 {
     const int64_t n = a.n_rows, wave = resident;
     a.tile_ahead = resident;
-    a.tail_rows = n <= wave * (kTile / 4) ? kTile / 4 : kTile / 2;
-    a.n_big = n <= wave * kTile ? 0 : (int32_t)(n / kTile - wave / 2);
-    return (unsigned)(a.n_big + (n - (int64_t)a.n_big * kTile + a.tail_rows - 1) / a.tail_rows);
+    a.big_rows = kTile;
+    a.tail_rows = kTile / 2;
+    a.n_big = 0;
+    if (n > wave * kTile) {
+        a.n_big = (int32_t)(n / kTile - wave / 2);
+    } else if (n <= wave * (kTile / 4)) {
+        a.tail_rows = kTile / 4;
+    } else if (n > wave * (kTile / 2) && 10 * n <= 7 * wave * kTile) {
+        a.big_rows = kTile / 2;
+        a.tail_rows = kTile / 4;
+        a.n_big = (int32_t)(3 * n / 4 / a.big_rows);
+    }
+    return (unsigned)(a.n_big + (n - (int64_t)a.n_big * a.big_rows + a.tail_rows - 1) / a.tail_rows);
 }
 
 // FP32: the visible rows of a tile whose items run together (768 SH items, then

@@ -409,10 +409,10 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_x(const StepAr
     constexpr int kNsh = 48 / kW;
     __shared__ TileListsX<kTile> L;
     pdl_enter();
-    prefetch_tile_ahead<kTile>(a, vis_src);
-    prefetch_tile_ahead_x<kTile>(a);
+    prefetch_tile_ahead(a, vis_src);
+    prefetch_tile_ahead_x(a);
     int nv, ni;
-    tile_decide_x<kTile, S::kRowBytes, S::kTByte>(a, vis_src, tile_span<kTile>(a, blockIdx.x), L, nv, ni);
+    tile_decide_x<kTile, S::kRowBytes, S::kTByte>(a, vis_src, tile_span(a, blockIdx.x), L, nv, ni);
 
     unsigned my_active = 0;
     constexpr int kSmall = kSmallItems<kPrec>, kOpItem = 11 + kSmall;     // the item holding the opacity

@@ -235,8 +235,8 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile(const StepArgs
 {
     __shared__ TileLists<kTile> L;
     pdl_enter();
-    prefetch_tile_ahead<kTile>(a, vis_src);
-    process_tile<kTile, kPrec, kW>(a, vis_src, tile_span<kTile>(a, blockIdx.x), L);
+    prefetch_tile_ahead(a, vis_src);
+    process_tile<kTile, kPrec, kW>(a, vis_src, tile_span(a, blockIdx.x), L);
 }
 
 // The terms form: the same step with the active count N_a (Sec. 4) and/or
@@ -248,9 +248,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_terms(const St
     __shared__ TileLists<kTile> L;
     __shared__ TileTerms<kTile> X;
     pdl_enter();
-    prefetch_tile_ahead<kTile>(a, vis_src);
-    prefetch_tile_ahead_x<kTile>(a);
-    process_tile<kTile, kPrec, kW, true>(a, vis_src, tile_span<kTile>(a, blockIdx.x), L, &X);
+    prefetch_tile_ahead(a, vis_src);
+    prefetch_tile_ahead_x(a);
+    process_tile<kTile, kPrec, kW, true>(a, vis_src, tile_span(a, blockIdx.x), L, &X);
 }
 
 // Tile t of a scene of a batch: kTile rows, the last one what is left.
