@@ -30,7 +30,7 @@ __global__ void __launch_bounds__(kThreads) visibility_kernel(const float *__res
 {
     __shared__ int32_t s_cnt[kThreads / 32];
     __shared__ unsigned long long s_base;
-    pdl_enter();
+    pdl_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t row = (int64_t)blockIdx.x * kThreads + tid;
     const float *c = cam.c;
@@ -56,13 +56,15 @@ __global__ void __launch_bounds__(kThreads) visibility_kernel(const float *__res
         off += __popc(b & ((1u << lane) - 1u));
         list[s_base + off] = (int32_t)row;
     }
+    pdl_release();
 }
 
 // The count starts from zero.  A kernel in the launch chain rather than a memset:
 // the filter's CTAs are then already resident when the zero is written.
 __global__ void zero_count_kernel(unsigned long long *count)
 {
-    pdl_enter();
+    pdl_release();
+    pdl_wait();
     *count = 0ull;
 }
 
@@ -81,7 +83,7 @@ __global__ void __launch_bounds__(kThreads) visibility4_kernel(const float *__re
 {
     __shared__ int32_t s_warp[kThreads / 32];
     __shared__ unsigned long long s_base;
-    pdl_enter();
+    pdl_wait();
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t r0 = ((int64_t)blockIdx.x * kThreads + tid) * kVisRpt;
     const float *c = cam.c;
@@ -134,6 +136,7 @@ __global__ void __launch_bounds__(kThreads) visibility4_kernel(const float *__re
         for (int j = 0; j < kVisRpt; ++j)
             if (vis & (1u << j)) *dst++ = (int32_t)(r0 + j);
     }
+    pdl_release();
 }
 
 // --------------------------------------------------------------- bias table
@@ -171,6 +174,7 @@ template <int kChunks, int kRowBytes>
 __global__ void reindex_kernel(const StateView in, int32_t n_in, const StateView out, int32_t n_out,
                                const int32_t *__restrict__ src, const uint8_t *__restrict__ reset, int32_t *err)
 {
+    pdl_wait();
     const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t j = gid / kChunks;
     const int c = (int)(gid - j * kChunks);
@@ -188,6 +192,7 @@ __global__ void reindex_kernel(const StateView in, int32_t n_in, const StateView
     }
     __stcs(reinterpret_cast<uint4 *>(static_cast<char *>(out.m) + (size_t)j * (2 * kRowBytes) + 16 * c), mv);
     __stcs(reinterpret_cast<uint4 *>(static_cast<char *>(out.v) + (size_t)j * (2 * kRowBytes) + 16 * c), vv);
+    pdl_release();
 }
 
 // ----------------------------------------------------------- attribute gather
@@ -229,6 +234,7 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const gs_attrs in, int
     __shared__ __align__(16) float sh[kGatherRows * 48], rot[kGatherRows * 4], xyz[kGatherRows * 3],
         scale[kGatherRows * 3], op[kGatherRows];
     __shared__ int32_t s_src[kGatherRows];
+    pdl_wait();
     const int tid = threadIdx.x;
     const int64_t r0 = (int64_t)blockIdx.x * kGatherRows;
     const int nrow = (int)min((int64_t)kGatherRows, (int64_t)n_new - r0);
@@ -259,6 +265,7 @@ __global__ void __launch_bounds__(kThreads) gather_kernel(const gs_attrs in, int
     gather_small_out<3>(out.xyz + r0 * 3, s_src, nrow, all, xyz);
     gather_small_out<3>(out.scale + r0 * 3, s_src, nrow, all, scale);
     gather_small_out<1>(out.opacity + r0, s_src, nrow, all, op);
+    pdl_release();
 }
 
 // ------------------------------------------------------------- row copy
@@ -296,7 +303,7 @@ __device__ __forceinline__ float4 xor4(float4 x, uint32_t b)
 
 __global__ void __launch_bounds__(kThreads) copy_rows_kernel(const CopyRowsArgs c)
 {
-    pdl_enter();
+    pdl_wait();
     const int64_t nl = c.nl, e_sh = 12 * nl, e_m = e_sh + (int64_t)c.chunks * nl, e_st = e_m + (int64_t)c.chunks * nl;
     const int64_t total = e_st + 4 * nl;
     for (int64_t w = (int64_t)blockIdx.x * kThreads + threadIdx.x; w < total; w += (int64_t)gridDim.x * kThreads) {
@@ -341,6 +348,7 @@ __global__ void __launch_bounds__(kThreads) copy_rows_kernel(const CopyRowsArgs 
             }
         }
     }
+    pdl_release();
 }
 
 // ------------------------------------------------------------ active rows
@@ -359,7 +367,7 @@ __global__ void __launch_bounds__(kThreads) active_count_kernel(const float *__r
                                                                 float tau_act, int32_t *__restrict__ blk)
 {
     __shared__ int32_t warp_sum[kActWarps];
-    pdl_enter();
+    pdl_wait();
     const int64_t r0 = (int64_t)blockIdx.x * kActRows;
     float x[kActRpt];
 #pragma unroll
@@ -378,6 +386,7 @@ __global__ void __launch_bounds__(kThreads) active_count_kernel(const float *__r
         for (int w = 0; w < kActWarps; ++w) s += warp_sum[w];
         blk[blockIdx.x] = s;
     }
+    pdl_release();
 }
 
 // rows == NULL: count only (only the last block runs, to write the total).
@@ -387,7 +396,7 @@ __global__ void __launch_bounds__(kThreads) active_write_kernel(const float *__r
 {
     __shared__ int32_t cnt[kActRpt * kActWarps];      // per (pass, warp), then its exclusive offset
     __shared__ int32_t part[kActWarps];
-    pdl_enter();
+    pdl_wait();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const bool last = blockIdx.x == gridDim.x - 1;
     if (!rows && !last) return;
@@ -440,6 +449,7 @@ __global__ void __launch_bounds__(kThreads) active_write_kernel(const float *__r
     for (int j = 0; j < kActRpt; ++j)
         if (bal[j] & (1u << lane))
             rows[cnt[j * kActWarps + warp] + __popc(bal[j] & lt)] = (int32_t)(r0 + j * kThreads + threadIdx.x);
+    pdl_release();
 }
 
 unsigned blocks_for(int64_t n_threads) { return (unsigned)((n_threads + kThreads - 1) / kThreads); }
@@ -469,6 +479,18 @@ cudaError_t launch_bias_table(double beta1, double beta2, int32_t len, double *t
     return cudaGetLastError();
 }
 
+namespace {
+
+template <int kChunks, int kRowBytes>
+cudaError_t launch_reindex_t(const StateView &in, int32_t n_in, const StateView &out, int32_t n_out, const int32_t *src,
+                             const uint8_t *reset, int32_t *err, cudaStream_t s)
+{
+    return launch_pdl(reindex_kernel<kChunks, kRowBytes>, blocks_for((int64_t)n_out * kChunks), kThreads, s, in, n_in,
+                      out, n_out, src, reset, err);
+}
+
+}  // namespace
+
 cudaError_t launch_reindex(const StateView &in, int32_t n_in, const StateView &out, int32_t n_out,
                            const int32_t *src, const uint8_t *reset, int32_t *err, cudaStream_t s)
 {
@@ -476,25 +498,12 @@ cudaError_t launch_reindex(const StateView &in, int32_t n_in, const StateView &o
     switch (in.prec) {
     case GS_MOM_FP8E4M3: return launch_reindex_fp8(in, n_in, out, n_out, src, reset, err, s);
     case GS_MOM_FP32:      // whole 256-B rows (the last 16 B are padding): a warp moves two rows
-        reindex_kernel<16, kRowBytesF32><<<blocks_for((int64_t)n_out * 16), kThreads, 0, s>>>(in, n_in, out, n_out,
-                                                                                             src, reset, err);
-        break;
-    case GS_MOM_BF16:
-        reindex_kernel<8, kRowBytesBf16><<<blocks_for((int64_t)n_out * 8), kThreads, 0, s>>>(in, n_in, out, n_out,
-                                                                                            src, reset, err);
-        break;
-    case GS_MOM_BF16_HYBRID:
-        reindex_kernel<10, kRowBytesHyb><<<blocks_for((int64_t)n_out * 10), kThreads, 0, s>>>(in, n_in, out, n_out,
-                                                                                             src, reset, err);
-        break;
-    case GS_MOM_FP16_BLOCK:
-        reindex_kernel<8, kRowBytesF16B><<<blocks_for((int64_t)n_out * 8), kThreads, 0, s>>>(in, n_in, out, n_out,
-                                                                                            src, reset, err);
-        break;
-    default:
-        return cudaErrorNotSupported;
+        return launch_reindex_t<16, kRowBytesF32>(in, n_in, out, n_out, src, reset, err, s);
+    case GS_MOM_BF16: return launch_reindex_t<8, kRowBytesBf16>(in, n_in, out, n_out, src, reset, err, s);
+    case GS_MOM_BF16_HYBRID: return launch_reindex_t<10, kRowBytesHyb>(in, n_in, out, n_out, src, reset, err, s);
+    case GS_MOM_FP16_BLOCK: return launch_reindex_t<8, kRowBytesF16B>(in, n_in, out, n_out, src, reset, err, s);
+    default: return cudaErrorNotSupported;
     }
-    return cudaGetLastError();
 }
 
 cudaError_t launch_gather_attrs(const gs_attrs &in, int32_t n_in, const gs_attrs &out, const int32_t *src,
@@ -502,8 +511,7 @@ cudaError_t launch_gather_attrs(const gs_attrs &in, int32_t n_in, const gs_attrs
 {
     if (n_new <= 0) return cudaSuccess;
     const unsigned grid = (unsigned)(((int64_t)n_new + kGatherRows - 1) / kGatherRows);
-    gather_kernel<<<grid, kThreads, 0, s>>>(in, n_in, out, src, n_new, err);
-    return cudaGetLastError();
+    return launch_pdl(gather_kernel, grid, kThreads, s, in, n_in, out, src, n_new, err);
 }
 
 cudaError_t launch_copy_rows(const gs_attrs &a, const gs_grads &g, void *m, int32_t row_bytes,

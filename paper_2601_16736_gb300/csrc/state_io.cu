@@ -212,6 +212,7 @@ __global__ void __launch_bounds__(kThreads) export_kernel(void *state, int32_t n
     static_assert(kIoRows * kC2 % kThreads == 0 && kPer % kU == 0, "whole chunks per thread");
     __shared__ __align__(16) float x[kIoV + kIoFloats];
     __shared__ uint32_t ts[kIoRows];
+    pdl_wait();
     const int tid = threadIdx.x;
     const int64_t r0 = (int64_t)blockIdx.x * kIoRows;
     const int nrow = (int)min((int64_t)kIoRows, (int64_t)n - r0);
@@ -247,6 +248,7 @@ __global__ void __launch_bounds__(kThreads) export_kernel(void *state, int32_t n
     if (m_out) store_canonical(m_out + r0 * kNumCols, nf, x);
     if (v_out) store_canonical(v_out + r0 * kNumCols, nf, x + kIoV);
     if (t_out && tid < nrow) t_out[r0 + tid] = ts[tid];
+    pdl_release();
 }
 
 // A part that is NULL keeps the stored one.
@@ -259,6 +261,7 @@ __global__ void __launch_bounds__(kThreads) import_kernel(void *state, int32_t n
     constexpr int kC2 = 2 * C::kChunks, kPer = kIoRows * kC2 / kThreads;
     __shared__ __align__(16) float x[kIoV + kIoFloats];
     __shared__ uint32_t ts[kIoRows];
+    pdl_wait();
     const int tid = threadIdx.x;
     const int64_t r0 = (int64_t)blockIdx.x * kIoRows;
     const int nrow = (int)min((int64_t)kIoRows, (int64_t)n - r0);
@@ -301,22 +304,21 @@ __global__ void __launch_bounds__(kThreads) import_kernel(void *state, int32_t n
                 reinterpret_cast<uint32_t *>(out + q)[kPrec == GS_MOM_BF16 ? 2 : 3] = ts[r];
         }
     }
+    pdl_release();
 }
 
 template <int kPrec>
 cudaError_t export_t(const StateView &st, int32_t n, float *m, float *v, uint32_t *t, cudaStream_t s)
 {
     const unsigned grid = (unsigned)(((int64_t)n + kIoRows - 1) / kIoRows);
-    export_kernel<kPrec><<<grid, kThreads, 0, s>>>(st.m, n, m, v, t);
-    return cudaGetLastError();
+    return launch_pdl(export_kernel<kPrec>, grid, kThreads, s, st.m, n, m, v, t);
 }
 
 template <int kPrec>
 cudaError_t import_t(const StateView &st, int32_t n, const float *m, const float *v, const uint32_t *t, cudaStream_t s)
 {
     const unsigned grid = (unsigned)(((int64_t)n + kIoRows - 1) / kIoRows);
-    import_kernel<kPrec><<<grid, kThreads, 0, s>>>(st.m, n, m, v, t);
-    return cudaGetLastError();
+    return launch_pdl(import_kernel<kPrec>, grid, kThreads, s, st.m, n, m, v, t);
 }
 
 }  // namespace

@@ -408,7 +408,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_x(const StepAr
     using S = State<kPrec>;
     constexpr int kNsh = 48 / kW;
     __shared__ TileListsX<kTile> L;
-    pdl_enter();
+    pdl_wait();
     prefetch_tile_ahead(a, vis_src);
     prefetch_tile_ahead_x(a);
     int nv, ni;
@@ -459,6 +459,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_x(const StepAr
         __syncthreads();
         if (threadIdx.x == 0 && L.active) atomicAdd(a.n_active, (unsigned long long)L.active);
     }
+    pdl_release();
 }
 
 }  // namespace

@@ -700,7 +700,7 @@ template <int kT, int kMinBlocks>
 __global__ void __launch_bounds__(kT, kMinBlocks) step_fp8_full(const StepArgs a, const int vis_src, const int full0)
 {
     __shared__ F8FullShared F;
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    pdl_release();
     f8_block_full<kT>(a, vis_src, full0 + (int)kF8FullEvery * (int)blockIdx.x, F);
 }
 
@@ -723,10 +723,12 @@ __global__ void __launch_bounds__(kT, kMinBlocks) step_fp8_grow(const StepArgs a
 {
     __shared__ F8GrowShared S;
     f8_grow_tile<kT>(a, vis_src, (int)blockIdx.x, full0, S);
-    if (blockIdx.x == gridDim.x - 1) asm volatile("griddepcontrol.wait;" ::: "memory");
+    if (blockIdx.x == gridDim.x - 1) pdl_wait();
 }
 
-// A scene of at most one wave: one launch, the n_full longer CTAs first.
+// A scene of at most one wave: one launch, the n_full longer CTAs first, in the
+// chain of programmatic launches (30 k rows, 88 % visible: 21.0 us against 23.3;
+// 30 %: 15.3 against 17.3).
 template <int kT, int kMinBlocks>
 __global__ void __launch_bounds__(kT, kMinBlocks) step_fp8(const StepArgs a, const int vis_src, const int full0,
                                                             const int n_full)
@@ -735,9 +737,11 @@ __global__ void __launch_bounds__(kT, kMinBlocks) step_fp8(const StepArgs a, con
         F8FullShared full;
         F8GrowShared grow;
     } sh;
+    pdl_wait();
     const int b = (int)blockIdx.x;
     if (b < n_full) f8_block_full<kT>(a, vis_src, full0 + (int)kF8FullEvery * b, sh.full);
     else f8_grow_tile<kT>(a, vis_src, b - n_full, full0, sh.grow);
+    pdl_release();
 }
 
 // ------------------------------------------------------ export / import
@@ -1007,15 +1011,12 @@ cudaError_t launch_step_fp8(const StepArgs &a, int vis_src, cudaStream_t s)
     // the tiles of this step's full pass: (iteration + tile) % kF8FullEvery == 0
     const int full0 = (int)((kF8FullEvery - (uint32_t)(a.k_ctr % kF8FullEvery)) % kF8FullEvery);
     const int n_full = full0 < n_tiles ? (n_tiles - full0 + (int)kF8FullEvery - 1) / (int)kF8FullEvery : 0;
-    if (n_tiles <= resident / 2) {
-        step_fp8<2 * kThreads, kF8MinBlocks / 2>
-            <<<(unsigned)(n_full + n_tiles), 2 * kThreads, 0, s>>>(b, vis_src, full0, n_full);
-        return cudaGetLastError();
-    }
-    if (n_tiles <= resident || !n_full) {
-        step_fp8<kThreads, kF8MinBlocks><<<(unsigned)(n_full + n_tiles), kThreads, 0, s>>>(b, vis_src, full0, n_full);
-        return cudaGetLastError();
-    }
+    if (n_tiles <= resident / 2)
+        return launch_pdl(step_fp8<2 * kThreads, kF8MinBlocks / 2>, (unsigned)(n_full + n_tiles), 2 * kThreads, s, b,
+                          vis_src, full0, n_full);
+    if (n_tiles <= resident || !n_full)
+        return launch_pdl(step_fp8<kThreads, kF8MinBlocks>, (unsigned)(n_full + n_tiles), kThreads, s, b, vis_src,
+                          full0, n_full);
     step_fp8_full<kThreads, kF8MinBlocks><<<(unsigned)n_full, kThreads, 0, s>>>(b, vis_src, full0);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

@@ -234,9 +234,10 @@ template <int kTile, int kMinBlocks, int kPrec, int kW>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile(const StepArgs a, const int vis_src)
 {
     __shared__ TileLists<kTile> L;
-    pdl_enter();
+    pdl_wait();
     prefetch_tile_ahead(a, vis_src);
     process_tile<kTile, kPrec, kW>(a, vis_src, tile_span(a, blockIdx.x), L);
+    pdl_release();
 }
 
 // The terms form: the same step with the active count N_a (Sec. 4) and/or
@@ -247,10 +248,11 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_terms(const St
 {
     __shared__ TileLists<kTile> L;
     __shared__ TileTerms<kTile> X;
-    pdl_enter();
+    pdl_wait();
     prefetch_tile_ahead(a, vis_src);
     prefetch_tile_ahead_x(a);
     process_tile<kTile, kPrec, kW, true>(a, vis_src, tile_span(a, blockIdx.x), L, &X);
+    pdl_release();
 }
 
 // Tile t of a scene of a batch: kTile rows, the last one what is left.
