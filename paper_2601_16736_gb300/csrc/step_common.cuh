@@ -19,6 +19,11 @@ __device__ __forceinline__ float4 ldg4_stream(const float *p)
 {
     return __ldcs(reinterpret_cast<const float4 *>(p));
 }
+// Gradients of a visible row: streamed (evict-first), or kept as ordinary lines.
+template <bool kKeep>
+__device__ __forceinline__ float4 ldg4(const float *p) { return kKeep ? ld4(p) : ldg4_stream(p); }
+template <bool kKeep>
+__device__ __forceinline__ float ldg1(const float *p) { return kKeep ? *p : __ldcs(p); }
 // results are not read again in this step: store them evict-first
 __device__ __forceinline__ void st4(float *p, float4 x) { __stcs(reinterpret_cast<float4 *>(p), x); }
 
@@ -445,7 +450,7 @@ struct State<GS_MOM_FP16_BLOCK> {
 // high half of the fourth word.  The visible update as small_item; RSR
 // scales the moments afterwards.  kX: item 13 subtracts the row's noise nz
 // from xyz and returns whether the row is active after the step.
-template <bool kX>
+template <bool kX, bool kKeep>
 __device__ __forceinline__ bool small_item_f16b(const StepArgs &a, const int32_t row, const int c, const bool sampled,
                                                 const float2 f, const float3 nz)
 {
@@ -460,7 +465,7 @@ __device__ __forceinline__ bool small_item_f16b(const StepArgs &a, const int32_t
         decode_w<4>(wv, dec_scale((uint8_t)vr[kF16BExp + 6]), v);
         float *pt = a.a_rot + r * 4;
         float4 th = ld4(pt);
-        const float4 g = ldg4_stream(a.g_rot + r * 4);
+        const float4 g = ldg4<kKeep>(a.g_rot + r * 4);
         const float l = a.lr[2];
         th.x = step_element(th.x, g.x, m[0], v[0], f.x, f.y, a, l, false, 0.f, 0.f, 0.f);
         th.y = step_element(th.y, g.y, m[1], v[1], f.x, f.y, a, l, false, 0.f, 0.f, 0.f);
@@ -491,8 +496,8 @@ __device__ __forceinline__ bool small_item_f16b(const StepArgs &a, const int32_t
         float *px = a.a_xyz + r * 3, *ps = a.a_scale + r * 3, *po = a.a_op + r;
         float x0 = px[0], x1 = px[1], x2 = px[2], s0 = ps[0], s1 = ps[1], s2 = ps[2], op = *po;
         const float *gx = a.g_xyz + r * 3, *gs = a.g_scale + r * 3;
-        const float g0 = __ldcs(gx), g1 = __ldcs(gx + 1), g2 = __ldcs(gx + 2);
-        const float gs0 = __ldcs(gs), gs1 = __ldcs(gs + 1), gs2 = __ldcs(gs + 2), go = __ldcs(a.g_op + r);
+        const float g0 = ldg1<kKeep>(gx), g1 = ldg1<kKeep>(gx + 1), g2 = ldg1<kKeep>(gx + 2);
+        const float gs0 = ldg1<kKeep>(gs), gs1 = ldg1<kKeep>(gs + 1), gs2 = ldg1<kKeep>(gs + 2), go = ldg1<kKeep>(a.g_op + r);
         const bool ds = a.dar_s != 0, dop = a.dar_o != 0;
         // regulariser derivatives at the old values (App. Eqs. scale, opacity)
         const float r0s = ds ? expf(s0) : 0.f, r1s = ds ? expf(s1) : 0.f, r2s = ds ? expf(s2) : 0.f;
@@ -707,7 +712,7 @@ constexpr int kSmallItems = kPrec == GS_MOM_FP16_BLOCK ? 2 : 3;
 
 // SH item i of a visible row: SH columns kW*i .. kW*i+kW-1 (0-2 are the DC
 // term, learning rate lr[4]; the rest lr[5]); no regulariser.
-template <int kPrec, int kW>
+template <int kPrec, int kW, bool kKeep = false>
 __device__ __forceinline__ void sh_item(const StepArgs &a, const int32_t row, const int i, const bool sampled,
                                         const float2 f)
 {
@@ -723,7 +728,7 @@ __device__ __forceinline__ void sh_item(const StepArgs &a, const int32_t row, co
         const size_t off = (size_t)row * 48 + kW * i;
 #pragma unroll
         for (int q = 0; q < kW / 4; ++q) {
-            const float4 y = ldg4_stream(a.g_sh + off + 4 * q);
+            const float4 y = ldg4<kKeep>(a.g_sh + off + 4 * q);
             const float gq[4] = {y.x, y.y, y.z, y.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -758,7 +763,7 @@ __device__ __forceinline__ void sh_item(const StepArgs &a, const int32_t row, co
     const size_t off = (size_t)row * 48 + kW * i;
 #pragma unroll
     for (int q = 0; q < kW / 4; ++q) {
-        const float4 x = ld4(a.a_sh + off + 4 * q), y = ldg4_stream(a.g_sh + off + 4 * q);
+        const float4 x = ld4(a.a_sh + off + 4 * q), y = ldg4<kKeep>(a.g_sh + off + 4 * q);
         th[4 * q] = x.x; th[4 * q + 1] = x.y; th[4 * q + 2] = x.z; th[4 * q + 3] = x.w;
         g[4 * q] = y.x; g[4 * q + 1] = y.y; g[4 * q + 2] = y.z; g[4 * q + 3] = y.w;
     }
@@ -827,12 +832,12 @@ __device__ __forceinline__ float3 noise_term(const StepArgs &a, int32_t row, flo
 // row's noise nz, and the opacity item returns whether the row is active
 // after the step (opacity logit above tau_act); otherwise nz is unused and
 // the result false.
-template <int kPrec, bool kX = false>
+template <int kPrec, bool kX = false, bool kKeep = false>
 __device__ __forceinline__ bool small_item(const StepArgs &a, const int32_t row, const int c, const bool sampled,
                                            const float2 f, const float3 nz = float3{0.f, 0.f, 0.f})
 {
     if constexpr (kPrec == GS_MOM_FP16_BLOCK) {
-        return small_item_f16b<kX>(a, row, c, sampled, f, nz);
+        return small_item_f16b<kX, kKeep>(a, row, c, sampled, f, nz);
     } else {
         bool active = false;
         using S = State<kPrec>;
@@ -843,7 +848,7 @@ __device__ __forceinline__ bool small_item(const StepArgs &a, const int32_t row,
             // rotation quaternion
             float *pt = a.a_rot + r * 4;
             float4 th = ld4(pt);
-            const float4 g = ldg4_stream(a.g_rot + r * 4);
+            const float4 g = ldg4<kKeep>(a.g_rot + r * 4);
             const float l = a.lr[2];
             th.x = step_element(th.x, g.x, m.x, v.x, f.x, f.y, a, l, false, 0.f, 0.f, 0.f);
             th.y = step_element(th.y, g.y, m.y, v.y, f.x, f.y, a, l, false, 0.f, 0.f, 0.f);
@@ -856,7 +861,7 @@ __device__ __forceinline__ bool small_item(const StepArgs &a, const int32_t row,
             float *ps = a.a_scale + r * 3;
             const float *gx = a.g_xyz + r * 3;
             float x0 = px[0], x1 = px[1], x2 = px[2], s0 = ps[0];
-            const float g0 = __ldcs(gx), g1 = __ldcs(gx + 1), g2 = __ldcs(gx + 2), gs0 = __ldcs(a.g_scale + r * 3);
+            const float g0 = ldg1<kKeep>(gx), g1 = ldg1<kKeep>(gx + 1), g2 = ldg1<kKeep>(gx + 2), gs0 = ldg1<kKeep>(a.g_scale + r * 3);
             const bool ds = a.dar_s != 0;
             // scale: dR/dkappa = exp(kappa) at the old value (App. Eq. scale)
             const float r0s = ds ? expf(s0) : 0.f;
@@ -875,7 +880,7 @@ __device__ __forceinline__ bool small_item(const StepArgs &a, const int32_t row,
             float *po = a.a_op + r;
             const float *gsp = a.g_scale + r * 3;
             float s1 = ps[1], s2 = ps[2], op = *po;
-            const float gs1 = __ldcs(gsp + 1), gs2 = __ldcs(gsp + 2), go = __ldcs(a.g_op + r);
+            const float gs1 = ldg1<kKeep>(gsp + 1), gs2 = ldg1<kKeep>(gsp + 2), go = ldg1<kKeep>(a.g_op + r);
             const bool ds = a.dar_s != 0, dop = a.dar_o != 0;
             const float r1s = ds ? expf(s1) : 0.f, r2s = ds ? expf(s2) : 0.f;
             // opacity: dR/dtau = sig'(tau) at the old value (App. Eq. opacity)

@@ -21,6 +21,8 @@
 // (State<kPrec>): all arithmetic is FP32.
 
 
+#include <type_traits>
+
 #include "step_common.cuh"
 
 namespace gs {
@@ -159,10 +161,11 @@ __device__ __forceinline__ void tile_decide(const StepArgs &a, const int vis_src
 // (nv, nr of them in L), grouped by kind: SH items, then small items (FP32:
 // group of rows by group of rows), then RSR.  kX: the xyz items draw the rows' noise
 // from the values kept in X and subtract it, the opacity items count the rows
-// active after the step, and the tile's count is added to a.n_active.
-template <int kTile, int kPrec, int kW, bool kX>
+// active after the step, and the tile's count is added to a.n_active.  kLarge:
+// the gradients of a sparse tile are read as ordinary lines (kLargeRows).
+template <int kTile, int kPrec, int kW, bool kX, bool kLarge>
 __device__ __forceinline__ void tile_items(const StepArgs &a, const TileLists<kTile> &L, TileTerms<kTile> *X,
-                                           const int nv, const int nr)
+                                           const int nv, const int nr, const int rows)
 {
     constexpr int kNsh = 48 / kW, kItems = kNsh + kSmallItems<kPrec>;
     // One flat item space, walked as three loops (SH items, small items, RSR
@@ -172,12 +175,13 @@ __device__ __forceinline__ void tile_items(const StepArgs &a, const TileLists<kT
     unsigned my_active = 0;
     int w = threadIdx.x;
     // the items of rows j0 .. j0+ng-1 of the list
-    auto run = [&](const int j0, const int ng) {
+    auto run = [&](auto keep, const int j0, const int ng) {
+        constexpr bool kKeep = decltype(keep)::value;
         const int e_sh = kNsh * ng, e_vis = kItems * ng;
         for (; w < e_sh; w += kThreads) {
             const int q = w / kNsh, i = w - q * kNsh, j = j0 + q;
             const int32_t e = L.list[j];
-            sh_item<kPrec, kW>(a, e & 0x7fffffff, i, e < 0, L.fac[j]);
+            sh_item<kPrec, kW, kKeep>(a, e & 0x7fffffff, i, e < 0, L.fac[j]);
         }
         for (; w < e_vis; w += kThreads) {
             const int q = w - e_sh;
@@ -189,17 +193,19 @@ __device__ __forceinline__ void tile_items(const StepArgs &a, const TileLists<kT
                     const float4 q4 = X->q[j], s4 = X->sko[j];
                     nz = noise_term(a, e & 0x7fffffff, q4, s4.x, s4.y, s4.z, s4.w);
                 }
-                my_active += small_item<kPrec, true>(a, e & 0x7fffffff, c, e < 0, L.fac[j], nz) ? 1u : 0u;
+                my_active += small_item<kPrec, true, kKeep>(a, e & 0x7fffffff, c, e < 0, L.fac[j], nz) ? 1u : 0u;
             } else {
-                small_item<kPrec>(a, e & 0x7fffffff, c, e < 0, L.fac[j]);
+                small_item<kPrec, false, kKeep>(a, e & 0x7fffffff, c, e < 0, L.fac[j]);
             }
         }
         if constexpr (kPrec == GS_MOM_FP32) w -= e_vis;
     };
-    if constexpr (kPrec == GS_MOM_FP32) {
-        for (int j0 = 0; j0 < nv; j0 += kGroupRows) run(j0, min(nv - j0, kGroupRows));
+    if (kLarge && 4 * nv <= rows) {
+        if constexpr (kLarge) run(std::true_type{}, 0, nv);
+    } else if constexpr (kPrec == GS_MOM_FP32) {
+        for (int j0 = 0; j0 < nv; j0 += kGroupRows) run(std::false_type{}, j0, min(nv - j0, kGroupRows));
     } else {
-        run(0, nv);
+        run(std::false_type{}, 0, nv);
     }
     const int e0 = kPrec == GS_MOM_FP32 ? 0 : kItems * nv, e_all = e0 + kItems * nr;
     for (; w < e_all; w += kThreads) {
@@ -218,7 +224,7 @@ __device__ __forceinline__ void tile_items(const StepArgs &a, const TileLists<kT
 }
 
 // One tile: phase A, then its items.
-template <int kTile, int kPrec, int kW, bool kX = false>
+template <int kTile, int kPrec, int kW, bool kX = false, bool kLarge = false>
 __device__ __forceinline__ void process_tile(const StepArgs &a, const int vis_src, const TileSpan span,
                                              TileLists<kTile> &L, TileTerms<kTile> *X = nullptr)
 {
@@ -227,23 +233,23 @@ __device__ __forceinline__ void process_tile(const StepArgs &a, const int vis_sr
     using S = State<kPrec>;
     int nv, nr;
     tile_decide<kTile, S::kRowBytes, S::kTByte, kX>(a, vis_src, span, L, X, nv, nr);
-    tile_items<kTile, kPrec, kW, kX>(a, L, X, nv, nr);
+    tile_items<kTile, kPrec, kW, kX, kLarge>(a, L, X, nv, nr, span.rows);
 }
 
-template <int kTile, int kMinBlocks, int kPrec, int kW>
+template <int kTile, int kMinBlocks, int kPrec, int kW, bool kLarge>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile(const StepArgs a, const int vis_src)
 {
     __shared__ TileLists<kTile> L;
     pdl_wait();
     prefetch_tile_ahead(a, vis_src);
-    process_tile<kTile, kPrec, kW>(a, vis_src, tile_span(a, blockIdx.x), L);
+    process_tile<kTile, kPrec, kW, false, kLarge>(a, vis_src, tile_span(a, blockIdx.x), L);
     pdl_release();
 }
 
 // The terms form: the same step with the active count N_a (Sec. 4) and/or
 // position noise on the visible rows (App. Eq. disentangled_mu).  AIU and
 // noise on every row take the extended kernel instead.
-template <int kTile, int kMinBlocks, int kPrec, int kW>
+template <int kTile, int kMinBlocks, int kPrec, int kW, bool kLarge>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_terms(const StepArgs a, const int vis_src)
 {
     __shared__ TileLists<kTile> L;
@@ -251,7 +257,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_terms(const St
     pdl_wait();
     prefetch_tile_ahead(a, vis_src);
     prefetch_tile_ahead_x(a);
-    process_tile<kTile, kPrec, kW, true>(a, vis_src, tile_span(a, blockIdx.x), L, &X);
+    process_tile<kTile, kPrec, kW, true, kLarge>(a, vis_src, tile_span(a, blockIdx.x), L, &X);
     pdl_release();
 }
 
@@ -350,15 +356,39 @@ namespace {
 template <int kPrec>
 constexpr int kTermsMinBlocks = (kPrec == GS_MOM_FP32 || kPrec == GS_MOM_BF16) ? 5 : 4;
 
-template <int kPrec, int kW, bool kX>
-cudaError_t launch_tiles(const StepArgs &a, int vis_src, cudaStream_t s)
+// Gradients are read once, so a step streams them (evict-first), which leaves
+// room in L2 for what the next step reads again.  In a scene of this many rows
+// nothing stays that long, and in a sparse tile of it the lines of the small
+// groups, each shared by the rows around a visible one, were gone before the
+// next item came for them: there (at most 25 % visible) they are read as ordinary
+// lines.  10 % visible, 6 M rows: FP32 248 us against 260, hybrid 223 against
+// 230; 20 %, 3 M: FP32 200 against 204, BF16 160 against 166; 1.5 M rows: 2-5 %
+// in these three formats; 1 M: level, smaller scenes 1-2 % slower, so they keep
+// a kernel without the second form.  The hybrid kernel spills a few words with it
+// (2 M rows, 88 % visible: 445 against 441; 20 %: 125 against 128), so it waits
+// for a size of which a view shows a small part; the FP16-block kernel spills too
+// (1 M rows, 88 %: 211.4 against 210.2), gains nothing at 20 % and stays with one.
+template <int kPrec>
+constexpr int64_t kLargeRows = kPrec == GS_MOM_BF16_HYBRID ? 3 << 20 : 3 << 19;
+
+template <int kPrec, int kW, bool kX, bool kLarge>
+cudaError_t launch_tiles_t(const StepArgs &a, int vis_src, cudaStream_t s)
 {
-    auto k = kX ? step_tile_terms<kStepTile, kTermsMinBlocks<kPrec>, kPrec, kW>
-                : step_tile<kStepTile, kStepMinBlocks<kPrec>, kPrec, kW>;
+    auto k = kX ? step_tile_terms<kStepTile, kTermsMinBlocks<kPrec>, kPrec, kW, kLarge>
+                : step_tile<kStepTile, kStepMinBlocks<kPrec>, kPrec, kW, kLarge>;
     static int s_res[64] = {};
     StepArgs b = a;
     const unsigned grid = plan_tiles<kStepTile>(b, resident_ctas(reinterpret_cast<const void *>(k), s_res));
     return launch_pdl(k, grid, kThreads, s, b, vis_src);
+}
+
+template <int kPrec, int kW, bool kX>
+cudaError_t launch_tiles(const StepArgs &a, int vis_src, cudaStream_t s)
+{
+    if constexpr (kPrec != GS_MOM_FP16_BLOCK) {
+        if (a.n_rows >= kLargeRows<kPrec> && !a.g_host) return launch_tiles_t<kPrec, kW, kX, true>(a, vis_src, s);
+    }
+    return launch_tiles_t<kPrec, kW, kX, false>(a, vis_src, s);
 }
 
 }  // namespace

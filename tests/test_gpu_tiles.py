@@ -67,6 +67,38 @@ def test_tiling_does_not_change_the_step(G, prec, waves, tile, extra):
         r.close()
 
 
+@pytest.mark.parametrize("prec", ["FP32", "BF16", "BF16_HYBRID"])
+def test_large_sparse_scene(G, prec):
+    """From 1.5 Mi rows on (hybrid: 3 Mi), the sparse tiles of a step (and of its
+    form with the active count) read their gradients another way: same results."""
+    n = (3 << (20 if prec == "BF16_HYBRID" else 19)) + 17
+    groups = synth.scene_blobs(n, 81, 40.0)
+    grads = synth.grads_rows(n, 82)
+    one, cut, terms = (GpuScene(groups, prec=getattr(G, "GS_MOM_" + prec)) for _ in range(3))
+    for r in (one, cut, terms):
+        r.set_grads(grads)
+    cam = synth.ring_cameras(10, (0.0,))[3]
+    batch = G.gs_batch_create([cut.h])
+    nvis = torch.zeros(1, dtype=torch.int64, device="cuda")
+    active = torch.zeros(1, dtype=torch.int64, device="cuda")
+    kw = dict(restate=True, restate_ratio=0.3, seed=5)
+    p = G.make_params(synth.lr_for_step(1, 10), 1, **kw)
+    one.step_camera(cam, p)
+    batch.set(0, G.make_attrs(cut.attrs), G.make_attrs(cut.grads), G.make_camera(cam), p)
+    G.gs_batch_step(batch, nvis)
+    terms.step_camera(cam, G.make_params(synth.lr_for_step(1, 10), 1, n_active=active, **kw))
+    assert 0 < int(nvis.item()) == int(one.nvis.item()) < n // 4
+    assert int(active.item()) == int((terms.attrs["opacity"] > np.float32(-np.log(254.0))).sum().item())
+    for r in (cut, terms):
+        for k in one.attrs:
+            assert torch.equal(r.attrs[k], one.attrs[k])
+        for a, b in zip(r.state(), one.state()):
+            assert a.tobytes() == b.tobytes()
+    batch.close()
+    for r in (one, cut, terms):
+        r.close()
+
+
 def test_fp8_block_width_does_not_change_the_step(G):
     """The same blocks in a scene small enough for 512 threads a block and in
     one with a block more, which takes 256."""
