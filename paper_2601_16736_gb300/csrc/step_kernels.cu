@@ -269,6 +269,35 @@ __device__ __forceinline__ TileSpan whole_tile(const StepArgs &a, const int t)
     return {first, (int)min((int64_t)kTile, (int64_t)a.n_rows - first)};
 }
 
+// Scene of tile t of a batch (the last whose first tile is <= t), by all lanes of
+// a warp: one load of the whole table instead of a chain of them.  ahead: the
+// scene of tile t2 as well, from the same values (-1 beyond the batch).
+static_assert(kMaxBatch == 64, "two scenes per lane");
+__device__ __forceinline__ int batch_scene(const BatchParams *__restrict__ p, const int t, const int t2, int &ahead)
+{
+    const int lane = threadIdx.x & 31;
+    const int a = p->tile_start[lane], b = p->tile_start[lane + 32], n = p->n_scenes, total = p->total_tiles;
+    const bool ina = lane < n, inb = lane + 32 < n;
+    const unsigned ca = __ballot_sync(0xffffffffu, ina && a <= t), cb = __ballot_sync(0xffffffffu, inb && b <= t);
+    const unsigned da = __ballot_sync(0xffffffffu, ina && a <= t2), db = __ballot_sync(0xffffffffu, inb && b <= t2);
+    ahead = t2 < total ? __popc(da) + __popc(db) - 1 : -1;
+    return __popc(ca) + __popc(cb) - 1;
+}
+
+// Ask L2 for the means of tile t2 of scene s, as prefetch_tile_ahead does.  With
+// the one-load scene search: 16 scenes (8.5 M rows) FP32 858.6 us a step against
+// 870.6, 24 scenes 632 against 643.
+template <int kTile>
+__device__ __forceinline__ void batch_prefetch(const BatchParams *__restrict__ p, const int s, const int t2)
+{
+    if (threadIdx.x != 0 || s < 0) return;
+    const float *xyz = p->args[s].a_xyz;
+    const int64_t first = (int64_t)(t2 - p->tile_start[s]) * kTile;
+    const int rows = (int)min((int64_t)kTile, (int64_t)p->args[s].n_rows - first) & ~15;
+    if (rows > 0 && ((uintptr_t)xyz & 15u) == 0)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(xyz + first * 3), "r"(rows * 12) : "memory");
+}
+
 // Many scenes in one persistent launch.  The scene table lives in device
 // memory (p); CTAs take the next tile of the whole batch from the work
 // counter (tile t belongs to the scene s with tile_start[s] <= t <
@@ -285,18 +314,16 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_batch(const BatchPa
     __shared__ StepArgs sa;
     __shared__ int s_tile;
     const int tid = threadIdx.x;
-    const int total = p->total_tiles, n_scenes = p->n_scenes;
+    const int total = p->total_tiles;
     int cur = -1;
     for (;;) {
         if (tid == 0) s_tile = (int)atomicAdd(work, 1u);
         __syncthreads();
         const int t = s_tile;
         if (t >= total) break;
-        int lo = 0, hi = n_scenes - 1;         // last scene whose first tile is <= t
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (p->tile_start[mid] <= t) lo = mid; else hi = mid - 1;
-        }
+        int ahead;
+        const int t2 = t + (int)gridDim.x, lo = batch_scene(p, t, t2, ahead);
+        batch_prefetch<kTile>(p, ahead, t2);
         if (lo != cur) {
             const uint32_t *src = reinterpret_cast<const uint32_t *>(&p->args[lo]);
             uint32_t *dst = reinterpret_cast<uint32_t *>(&sa);
@@ -326,14 +353,14 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_batch_grid(const Ba
     __shared__ StepArgs sa;
     const int t = (int)blockIdx.x;
     if (t >= p->total_tiles) return;
-    int lo = 0, hi = p->n_scenes - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (p->tile_start[mid] <= t) lo = mid; else hi = mid - 1;
-    }
+    int sms, ahead;
+    asm("mov.u32 %0, %%nsmid;" : "=r"(sms));
+    const int t2 = t + kMinBlocks * sms;       // the tile that takes this one's place
+    const int lo = batch_scene(p, t, t2, ahead);
     const uint32_t *src = reinterpret_cast<const uint32_t *>(&p->args[lo]);
     uint32_t *dst = reinterpret_cast<uint32_t *>(&sa);
     for (int q = threadIdx.x; q < (int)(sizeof(StepArgs) / 4); q += kThreads) dst[q] = src[q];
+    batch_prefetch<kTile>(p, ahead, t2);
     __syncthreads();
     process_tile<kTile, kPrec, kW>(sa, kVisCamera, whole_tile<kTile>(sa, t - p->tile_start[lo]), L);
 }
