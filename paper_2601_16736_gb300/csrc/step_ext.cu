@@ -182,7 +182,7 @@ __device__ __forceinline__ bool small_item_x_f16b(const StepArgs &a, const int32
 // otherwise kFAiu: the AIU step from the current moments.  kFRsr scales the
 // moments afterwards; chunk 13 subtracts the row's noise `nz` from xyz.
 // Chunk 14 returns whether the row is active after the step.
-template <int kPrec>
+template <int kPrec, bool kKeep = false>
 __device__ __forceinline__ bool small_item_x(const StepArgs &a, const int32_t row, const int c, const bool vis,
                                              const uint8_t fl, const float2 f, const float3 nz)
 {
@@ -201,7 +201,7 @@ __device__ __forceinline__ bool small_item_x(const StepArgs &a, const int32_t ro
             float4 th = ld4(pt);
             const float l = a.lr[2];
             if (vis) {
-                const float4 g = ldg4_stream(a.g_rot + r * 4);
+                const float4 g = ldg4<kKeep>(a.g_rot + r * 4);
                 th.x = step_element(th.x, g.x, m.x, v.x, f.x, f.y, a, l, false, 0.f, 0.f, 0.f);
                 th.y = step_element(th.y, g.y, m.y, v.y, f.x, f.y, a, l, false, 0.f, 0.f, 0.f);
                 th.z = step_element(th.z, g.z, m.z, v.z, f.x, f.y, a, l, false, 0.f, 0.f, 0.f);
@@ -221,7 +221,7 @@ __device__ __forceinline__ bool small_item_x(const StepArgs &a, const int32_t ro
         float x0 = px[0], x1 = px[1], x2 = px[2], s0 = ps[0];
         if (vis) {
             const float *gx = a.g_xyz + r * 3;
-            const float g0 = __ldcs(gx), g1 = __ldcs(gx + 1), g2 = __ldcs(gx + 2), gs0 = __ldcs(a.g_scale + r * 3);
+            const float g0 = ldg1<kKeep>(gx), g1 = ldg1<kKeep>(gx + 1), g2 = ldg1<kKeep>(gx + 2), gs0 = ldg1<kKeep>(a.g_scale + r * 3);
             const bool ds = a.dar_s != 0;
             const float r0s = ds ? expf(s0) : 0.f;
             x0 = step_element(x0, g0, m.x, v.x, f.x, f.y, a, a.lr[0], false, 0.f, 0.f, 0.f);
@@ -245,7 +245,7 @@ __device__ __forceinline__ bool small_item_x(const StepArgs &a, const int32_t ro
         float s1 = ps[1], s2 = ps[2], op = *po;
         if (vis) {
             const float *gsp = a.g_scale + r * 3;
-            const float gs1 = __ldcs(gsp + 1), gs2 = __ldcs(gsp + 2), go = __ldcs(a.g_op + r);
+            const float gs1 = ldg1<kKeep>(gsp + 1), gs2 = ldg1<kKeep>(gsp + 2), go = ldg1<kKeep>(a.g_op + r);
             const bool ds = a.dar_s != 0, dop = a.dar_o != 0;
             const float r1s = ds ? expf(s1) : 0.f, r2s = ds ? expf(s2) : 0.f;
             const float rop = dop ? dsigmoid(op) : 0.f;
@@ -401,7 +401,7 @@ __device__ __forceinline__ void tile_decide_x(const StepArgs &a, const int vis_s
     __syncthreads();
 }
 
-template <int kTile, int kMinBlocks, int kPrec, int kW>
+template <int kTile, int kMinBlocks, int kPrec, int kW, bool kLarge>
 __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_x(const StepArgs a, const int vis_src)
 {
     static_assert(kTile % kThreads == 0, "tile must be a multiple of the block");
@@ -411,8 +411,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_x(const StepAr
     pdl_wait();
     prefetch_tile_ahead(a, vis_src);
     prefetch_tile_ahead_x(a);
+    const TileSpan span = tile_span(a, blockIdx.x);
     int nv, ni;
-    tile_decide_x<kTile, S::kRowBytes, S::kTByte>(a, vis_src, tile_span(a, blockIdx.x), L, nv, ni);
+    tile_decide_x<kTile, S::kRowBytes, S::kTByte>(a, vis_src, span, L, nv, ni);
 
     unsigned my_active = 0;
     constexpr int kSmall = kSmallItems<kPrec>, kOpItem = 11 + kSmall;     // the item holding the opacity
@@ -423,24 +424,27 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_x(const StepAr
     // share a loop body, so their register demands do not add up.
     int w = threadIdx.x;
     // the items of visible rows j0 .. j0+ng-1 of the list
-    auto run = [&](const int j0, const int ng) {
+    auto run = [&](auto keep, const int j0, const int ng) {
+        constexpr bool kKeep = decltype(keep)::value;
         const int e_sh = kNsh * ng, e_vis = (kNsh + kSmall) * ng;
         for (; w < e_sh; w += kThreads) {
             const int q = w / kNsh, i = w - q * kNsh, j = j0 + q;
-            sh_item<kPrec, kW>(a, L.list[j], i, (L.vflag[j] & kFRsr) != 0, L.fac[j]);
+            sh_item<kPrec, kW, kKeep>(a, L.list[j], i, (L.vflag[j] & kFRsr) != 0, L.fac[j]);
         }
         for (; w < e_vis; w += kThreads) {
             const int q = w - e_sh;
             const int j = j0 + q % ng, c = 12 + q / ng;
-            const bool act = small_item_x<kPrec>(a, L.list[j], c, true, L.vflag[j], L.fac[j], L.nz[j]);
+            const bool act = small_item_x<kPrec, kKeep>(a, L.list[j], c, true, L.vflag[j], L.fac[j], L.nz[j]);
             my_active += (c == kOpItem && act) ? 1u : 0u;
         }
         if constexpr (kPrec == GS_MOM_FP32) w -= e_vis;
     };
-    if constexpr (kPrec == GS_MOM_FP32) {
-        for (int j0 = 0; j0 < nv; j0 += kGroupRows) run(j0, min(nv - j0, kGroupRows));
+    if (kLarge && 4 * nv <= span.rows) {       // kLargeRows
+        if constexpr (kLarge) run(std::true_type{}, 0, nv);
+    } else if constexpr (kPrec == GS_MOM_FP32) {
+        for (int j0 = 0; j0 < nv; j0 += kGroupRows) run(std::false_type{}, j0, min(nv - j0, kGroupRows));
     } else {
-        run(0, nv);
+        run(std::false_type{}, 0, nv);
     }
     for (; w < e_ish; w += kThreads) {
         const int q = w - e0;
@@ -473,14 +477,27 @@ constexpr int kExtMinBlocks = (kPrec == GS_MOM_FP32 || kPrec == GS_MOM_BF16) ? 5
 
 namespace {
 
-template <int kPrec, int kW>
-cudaError_t launch_ext_t(const StepArgs &a, int vis_src, cudaStream_t s)
+template <int kPrec, int kW, bool kLarge>
+cudaError_t launch_ext_tiles(const StepArgs &a, int vis_src, cudaStream_t s)
 {
-    auto k = step_tile_x<kExtTile, kExtMinBlocks<kPrec>, kPrec, kW>;
+    auto k = step_tile_x<kExtTile, kExtMinBlocks<kPrec>, kPrec, kW, kLarge>;
     static int s_res[64] = {};
     StepArgs b = a;
     const unsigned grid = plan_tiles<kExtTile>(b, resident_ctas(reinterpret_cast<const void *>(k), s_res));
     return launch_pdl(k, grid, kThreads, s, b, vis_src);
+}
+
+// Large scenes as in the plain step (kLargeRows).  Noise on every row, FP32, 10 %
+// visible: 6 M rows 304.6 us against 312.4, 3 M 164.9 against 169.2; AIU, hybrid,
+// 4 M: 267 against 271; 30 % and 88 %: level.  BF16 loses by it here (3 M, 20 %:
+// 202 against 199).
+template <int kPrec, int kW>
+cudaError_t launch_ext_t(const StepArgs &a, int vis_src, cudaStream_t s)
+{
+    if constexpr (kPrec == GS_MOM_FP32 || kPrec == GS_MOM_BF16_HYBRID) {
+        if (a.n_rows >= kLargeRows<kPrec> && !a.g_host) return launch_ext_tiles<kPrec, kW, true>(a, vis_src, s);
+    }
+    return launch_ext_tiles<kPrec, kW, false>(a, vis_src, s);
 }
 
 }  // namespace

@@ -20,9 +20,6 @@
 // one item, once.  The storage format of the moments is a template parameter
 // (State<kPrec>): all arithmetic is FP32.
 
-
-#include <type_traits>
-
 #include "step_common.cuh"
 
 namespace gs {
@@ -382,21 +379,6 @@ namespace {
 // without spills (FP32, BF16), 4 for the hybrid and FP16-block formats.
 template <int kPrec>
 constexpr int kTermsMinBlocks = (kPrec == GS_MOM_FP32 || kPrec == GS_MOM_BF16) ? 5 : 4;
-
-// Gradients are read once, so a step streams them (evict-first), which leaves
-// room in L2 for what the next step reads again.  In a scene of this many rows
-// nothing stays that long, and in a sparse tile of it the lines of the small
-// groups, each shared by the rows around a visible one, were gone before the
-// next item came for them: there (at most 25 % visible) they are read as ordinary
-// lines.  10 % visible, 6 M rows: FP32 248 us against 260, hybrid 223 against
-// 230; 20 %, 3 M: FP32 200 against 204, BF16 160 against 166; 1.5 M rows: 2-5 %
-// in these three formats; 1 M: level, smaller scenes 1-2 % slower, so they keep
-// a kernel without the second form.  The hybrid kernel spills a few words with it
-// (2 M rows, 88 % visible: 445 against 441; 20 %: 125 against 128), so it waits
-// for a size of which a view shows a small part; the FP16-block kernel spills too
-// (1 M rows, 88 %: 211.4 against 210.2), gains nothing at 20 % and stays with one.
-template <int kPrec>
-constexpr int64_t kLargeRows = kPrec == GS_MOM_BF16_HYBRID ? 3 << 20 : 3 << 19;
 
 template <int kPrec, int kW, bool kX, bool kLarge>
 cudaError_t launch_tiles_t(const StepArgs &a, int vis_src, cudaStream_t s)

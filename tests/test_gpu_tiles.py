@@ -69,8 +69,8 @@ def test_tiling_does_not_change_the_step(G, prec, waves, tile, extra):
 
 @pytest.mark.parametrize("prec", ["FP32", "BF16", "BF16_HYBRID"])
 def test_large_sparse_scene(G, prec):
-    """From 1.5 Mi rows on (hybrid: 3 Mi), the sparse tiles of a step (and of its
-    form with the active count) read their gradients another way: same results."""
+    """From 1.5 Mi rows on (hybrid: 3 Mi), the sparse tiles of a step, and of its
+    forms with the optional terms, read their gradients another way: same results."""
     n = (3 << (20 if prec == "BF16_HYBRID" else 19)) + 17
     groups = synth.scene_blobs(n, 81, 40.0)
     grads = synth.grads_rows(n, 82)
@@ -89,11 +89,16 @@ def test_large_sparse_scene(G, prec):
     terms.step_camera(cam, G.make_params(synth.lr_for_step(1, 10), 1, n_active=active, **kw))
     assert 0 < int(nvis.item()) == int(one.nvis.item()) < n // 4
     assert int(active.item()) == int((terms.attrs["opacity"] > np.float32(-np.log(254.0))).sum().item())
-    for r in (cut, terms):
-        for k in one.attrs:
-            assert torch.equal(r.attrs[k], one.attrs[k])
-        for a, b in zip(r.state(), one.state()):
-            assert a.tobytes() == b.tobytes()
+    def same(r):
+        assert all(torch.equal(r.attrs[k], one.attrs[k]) for k in one.attrs)
+        assert all(a.tobytes() == b.tobytes() for a, b in zip(r.state(), one.state()))
+
+    same(cut)
+    same(terms)
+    # the form with noise on every row, here of size zero
+    one.step_camera(cam, G.make_params(synth.lr_for_step(2, 10), 2))
+    terms.step_camera(cam, G.make_params(synth.lr_for_step(2, 10), 2, noise=2, noise_lr=0.0))
+    same(terms)
     batch.close()
     for r in (one, cut, terms):
         r.close()
