@@ -660,18 +660,21 @@ __device__ __forceinline__ void prefetch_tile_ahead_x(const StepArgs &a)
 __device__ __forceinline__ bool sparse_tile(int nv, int rows) { return 5 * nv <= 3 * rows; }
 
 // The grid of a step over a.n_rows rows in CTAs of up to kTile rows, `resident`
-// of them at once, and its tile sizes (a.n_big, a.tail_rows).  A tile of 256
+// of them at once (0: not known), and its tile sizes (a.n_big, a.tail_rows).  A tile of 256
 // rows is the best size for a large sparse scene (128: 1.1-1.3 times the time
 // at 10-20 % visible, where a tile's items no longer fill its threads).  But a
 // scene that makes fewer tiles than the chip holds leaves it idle, and a large
 // one ends in a wave that is partly empty:
-//   * up to one wave of 256-row tiles, 128 rows to a CTA, and up to one wave
-//     of 64-row tiles, 64 rows (FP32, 88 % visible: 20 k rows 9.6 us against
-//     14.8, 190 k 52.6 against 60; 30 % visible: 20 k rows 9.3 against 9.8,
-//     190 k level);
-//   * of those, what makes 1 to 1.4 waves of 128 rows ends in a quarter of its
-//     rows by 64 (100 k rows, 88 % visible: 24.2 us against 27.8 for 128 rows
-//     throughout and 33.1 for 256; 30 % visible: level, and 16.9 for 256);
+//   * up to one wave of 64-row tiles, 64 rows to a CTA, and up to one wave of
+//     128-row tiles, 128 (FP32, 88 % visible: 20 k rows 9.6 us against 14.8 with
+//     256; 30 %: 9.3 against 9.8);
+//   * up to one wave of 256-row tiles, as many rows as make one wave (a multiple of
+//     16).  Sparse tiles take much the same time whatever their rows, so more than
+//     a wave of smaller ones costs what the second wave does, while dense ones gain
+//     little by it (FP32, 100 k rows: 10 % visible 7.3 us against 9.0 with 128-row
+//     tiles ending in 64-row ones, 88 % 22.4 against 22.2 and against 25.3 with 256;
+//     170 k: 9.0 against 11.7 with 128, 49.2 against 46.0; BF16, 120 k: 7.6
+//     against 10.4, 22.9 against 22.7);
 //   * beyond, the rows of the last half wave in 128-row tiles (1 M rows, 30 %
 //     visible: FP32 108.9 us against 109.9, BF16 at 777 k 66.6 against 68.0;
 //     88 % visible: FP32 279.7 against 285.7; 3 M and 6 M rows level).
@@ -687,10 +690,8 @@ inline unsigned plan_tiles(StepArgs &a, const int resident)
         a.n_big = (int32_t)(n / kTile - wave / 2);
     } else if (n <= wave * (kTile / 4)) {
         a.tail_rows = kTile / 4;
-    } else if (n > wave * (kTile / 2) && 10 * n <= 7 * wave * kTile) {
-        a.big_rows = kTile / 2;
-        a.tail_rows = kTile / 4;
-        a.n_big = (int32_t)(3 * n / 4 / a.big_rows);
+    } else if (n > wave * (kTile / 2)) {
+        a.tail_rows = (int32_t)((n + 16 * wave - 1) / (16 * wave) * 16);
     }
     return (unsigned)(a.n_big + (n - (int64_t)a.n_big * a.big_rows + a.tail_rows - 1) / a.tail_rows);
 }
