@@ -660,11 +660,11 @@ __device__ __forceinline__ void prefetch_tile_ahead_x(const StepArgs &a)
 __device__ __forceinline__ bool sparse_tile(int nv, int rows) { return 5 * nv <= 3 * rows; }
 
 // The grid of a step over a.n_rows rows in CTAs of up to kTile rows, `resident`
-// of them at once (0: not known), and its tile sizes (a.n_big, a.tail_rows).  A tile of 256
-// rows is the best size for a large sparse scene (128: 1.1-1.3 times the time
-// at 10-20 % visible, where a tile's items no longer fill its threads).  But a
-// scene that makes fewer tiles than the chip holds leaves it idle, and a large
-// one ends in a wave that is partly empty:
+// of them at once (0: not known), and its tile sizes (a.n_big, a.tail_rows).  A
+// tile of 256 rows is the best size for a large sparse scene (128: 1.1-1.3 times
+// the time at 10-20 % visible, where a tile's items no longer fill its threads).
+// But a scene that makes fewer tiles than the chip holds leaves it idle, and a
+// large one ends in a wave that is partly empty:
 //   * up to one wave of 64-row tiles, 64 rows to a CTA, and up to one wave of
 //     128-row tiles, 128 (FP32, 88 % visible: 20 k rows 9.6 us against 14.8 with
 //     256; 30 %: 9.3 against 9.8);
@@ -675,10 +675,18 @@ __device__ __forceinline__ bool sparse_tile(int nv, int rows) { return 5 * nv <=
 //     tiles ending in 64-row ones, 88 % 22.4 against 22.2 and against 25.3 with 256;
 //     170 k: 9.0 against 11.7 with 128, 49.2 against 46.0; BF16, 120 k: 7.6
 //     against 10.4, 22.9 against 22.7);
-//   * beyond, the rows of the last half wave in 128-row tiles (1 M rows, 30 %
-//     visible: FP32 108.9 us against 109.9, BF16 at 777 k 66.6 against 68.0;
-//     88 % visible: FP32 279.7 against 285.7; 3 M and 6 M rows level).
-template <int kTile>
+//   * beyond, the rows of the last eighth of a wave in 128-row tiles: dense scenes
+//     gain by every such tile, sparse ones lose by it.  With half a wave, a quarter
+//     and an eighth the step takes 0.96, 0.96 and 0.98 of its time with whole tiles
+//     only (777 k rows, 88 % visible, FP32; BF16 0.94, 0.94, 0.97) and, at 10 %,
+//     1.02, 1.00, 1.00 (BF16 1.03, 1.01, 1.01), but at 1.5 waves 1.03, 1.00, 0.99
+//     (300 k; BF16 1.07, 1.04, 1.02) and at 1.9 waves 1.05, 1.04, 1.01 (375 k; BF16
+//     1.08, 1.05, 1.02).
+//     kTerms: the kernels with optional terms have a longer phase A, and a sparse
+//     view pays for each wave of CTAs as such: the tail takes no more tiles than the
+//     last wave has room for (10 % visible, noise on visible rows, FP32: an eighth
+//     that begins another wave costs 1.13 at 375 k rows and 1.06 at 575 k).
+template <int kTile, bool kTerms>
 inline unsigned plan_tiles(StepArgs &a, const int resident)
 {
     const int64_t n = a.n_rows, wave = resident;
@@ -686,8 +694,13 @@ inline unsigned plan_tiles(StepArgs &a, const int resident)
     a.big_rows = kTile;
     a.tail_rows = kTile / 2;
     a.n_big = 0;
-    if (n > wave * kTile) {
-        a.n_big = (int32_t)(n / kTile - wave / 2);
+    if (wave <= 0) {
+        a.tail_rows = kTile;
+    } else if (n > wave * kTile) {
+        const int64_t last = ((n + kTile - 1) / kTile - 1) % wave + 1;      // whole tiles of the last wave
+        const int64_t cut = kTerms ? std::min(wave / 8, wave - 1 - last) : wave / 8;
+        if (cut > 0) a.n_big = (int32_t)(n / kTile - cut);
+        else a.tail_rows = kTile;
     } else if (n <= wave * (kTile / 4)) {
         a.tail_rows = kTile / 4;
     } else if (n > wave * (kTile / 2)) {

@@ -483,7 +483,7 @@ cudaError_t launch_ext_tiles(const StepArgs &a, int vis_src, cudaStream_t s)
     auto k = step_tile_x<kExtTile, kExtMinBlocks<kPrec>, kPrec, kW, kLarge>;
     static int s_res[64] = {};
     StepArgs b = a;
-    const unsigned grid = plan_tiles<kExtTile>(b, resident_ctas(reinterpret_cast<const void *>(k), s_res));
+    const unsigned grid = plan_tiles<kExtTile, true>(b, resident_ctas(reinterpret_cast<const void *>(k), s_res));
     return launch_pdl(k, grid, kThreads, s, b, vis_src);
 }
 

@@ -387,7 +387,7 @@ cudaError_t launch_tiles_t(const StepArgs &a, int vis_src, cudaStream_t s)
                 : step_tile<kStepTile, kStepMinBlocks<kPrec>, kPrec, kW, kLarge>;
     static int s_res[64] = {};
     StepArgs b = a;
-    const unsigned grid = plan_tiles<kStepTile>(b, resident_ctas(reinterpret_cast<const void *>(k), s_res));
+    const unsigned grid = plan_tiles<kStepTile, kX>(b, resident_ctas(reinterpret_cast<const void *>(k), s_res));
     return launch_pdl(k, grid, kThreads, s, b, vis_src);
 }
 

@@ -1,6 +1,7 @@
 """The tiles that a step is cut into (plan_tiles, tile_span), on the CPU: the
 host part of csrc/step_common.cuh compiled into a small program that prints, for
-a number of rows and of CTAs resident at once, the grid and every tile."""
+a number of rows and of CTAs resident at once, the grid and its tile sizes, for
+the plain step and for the one with optional terms."""
 import subprocess
 
 import pytest
@@ -16,7 +17,9 @@ int main(int argc, char **argv)
     for (int i = 1; i + 1 < argc; i += 2) {
         gs::StepArgs a = {};
         a.n_rows = atoi(argv[i]);
-        const unsigned grid = gs::plan_tiles<256>(a, atoi(argv[i + 1]));
+        unsigned grid = gs::plan_tiles<256, false>(a, atoi(argv[i + 1]));
+        std::printf("%u %d %d %d\n", grid, a.n_big, a.big_rows, a.tail_rows);
+        grid = gs::plan_tiles<256, true>(a, atoi(argv[i + 1]));
         std::printf("%u %d %d %d\n", grid, a.n_big, a.big_rows, a.tail_rows);
     }
 }
@@ -33,7 +36,8 @@ def plans(tmp_path_factory):
     def run(cases):
         out = subprocess.run([str(d / "plan"), *[str(x) for c in cases for x in c]], check=True, capture_output=True,
                              text=True).stdout
-        return [tuple(map(int, line.split())) for line in out.splitlines()]
+        got = [tuple(map(int, line.split())) for line in out.splitlines()]
+        return [(n, terms, *got[2 * i + terms]) for i, (n, _) in enumerate(cases) for terms in (0, 1)]
 
     return run
 
@@ -46,8 +50,7 @@ def _sizes(wave):
 
 @pytest.mark.parametrize("wave", [0, 1, 3, 608, 760])
 def test_tiles_cover_the_rows_once(plans, wave):
-    sizes = _sizes(wave)
-    for n, (grid, n_big, big, tail) in zip(sizes, plans([(n, wave) for n in sizes])):
+    for n, _, grid, n_big, big, tail in plans([(n, wave) for n in _sizes(wave)]):
         assert 0 < tail <= 256 and 0 < big <= 256 and tail % 16 == 0 and big % 16 == 0
         left = n - n_big * big                     # the rows of the tail_rows tiles
         assert n_big >= 0 and left >= 0
@@ -55,7 +58,14 @@ def test_tiles_cover_the_rows_once(plans, wave):
 
 
 @pytest.mark.parametrize("wave", [608, 760])
-def test_one_wave_of_whole_tiles_stays_one_wave(plans, wave):
-    sizes = [n for n in _sizes(wave) if n <= wave * 256]
-    for n, (grid, *_) in zip(sizes, plans([(n, wave) for n in sizes])):
-        assert grid <= wave
+def test_no_more_waves_than_whole_tiles(plans, wave):
+    """A sparse tile takes much the same time whatever its rows: up to one wave
+    of whole tiles, and beyond it with the optional terms, smaller tiles may fill
+    the last wave but not begin another; the plain step adds at most an eighth
+    of a wave."""
+    for n, terms, grid, *_ in plans([(n, wave) for n in _sizes(wave)]):
+        whole = -(-n // 256)
+        if terms or whole <= wave:
+            assert -(-grid // wave) == -(-whole // wave)
+        else:
+            assert grid <= whole + wave // 8 + 1
