@@ -709,13 +709,19 @@ inline unsigned plan_tiles(StepArgs &a, const int resident)
     return (unsigned)(a.n_big + (n - (int64_t)a.n_big * a.big_rows + a.tail_rows - 1) / a.tail_rows);
 }
 
-// FP32: the visible rows of a tile whose items run together (768 SH items, then
-// their small items) before the next rows'.  A row's last moment line holds both
-// SH and small columns, so the two should follow each other while the line is
+// FP32: the visible rows of a dense tile whose items run together (768 SH items,
+// then their small items) before the next rows'.  A row's last moment line holds
+// both SH and small columns, so the two should follow each other while the line is
 // in L2; with the tiles in flight of a dense scene larger than L2, it came and
-// went twice (1 M rows, 88 % visible: 269 us against 285; 30 %: level).  The
-// 16-bit formats take the whole tile as one group: the loop over groups costs
-// them registers (BF16, 30 % visible: 78 us against 68).
+// went twice (1 M rows, 88 % visible: 269 us against 285).  A tile with no more
+// than two groups runs as one: the loop over groups costs registers and gains
+// nothing there (10 % visible, 300 k rows: 14.0 us against 14.5; 20 %, 190 k: 12.8
+// against 13.5; 30 %, 150 k with noise on visible rows: 1.08 times the speed).  Not
+// in the kernels of large scenes, whose sparse tiles have a loop of their own (a
+// third one slowed them: AIU and noise, 2 M, 10 %: 150 us against 147), nor in the
+// batched ones, which spill with it (20 scenes of 8 k to 60 k rows: 1.02 times the
+// time).  The 16-bit formats take every tile as one group: the loop costs them more
+// (BF16, 30 % visible: 78 us against 68).
 constexpr int kGroupRows = 64;
 
 // Gradients are read once, so a step streams them (evict-first), which leaves

@@ -441,9 +441,9 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_x(const StepAr
     };
     if (kLarge && 4 * nv <= span.rows) {       // kLargeRows
         if constexpr (kLarge) run(std::true_type{}, 0, nv);
-    } else if constexpr (kPrec == GS_MOM_FP32) {
+    } else if (kPrec == GS_MOM_FP32 && (kLarge || nv > 2 * kGroupRows)) {
         for (int j0 = 0; j0 < nv; j0 += kGroupRows) run(std::false_type{}, j0, min(nv - j0, kGroupRows));
-    } else {
+    } else if constexpr (kPrec != GS_MOM_FP32 || !kLarge) {
         run(std::false_type{}, 0, nv);
     }
     for (; w < e_ish; w += kThreads) {

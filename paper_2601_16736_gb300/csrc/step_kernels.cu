@@ -155,12 +155,13 @@ __device__ __forceinline__ void tile_decide(const StepArgs &a, const int vis_src
 // ---------------------------------------------------------------- the kernel
 
 // Phase B of one tile: the items of its visible and invisible-sampled rows
-// (nv, nr of them in L), grouped by kind: SH items, then small items (FP32:
+// (nv, nr of them in L), grouped by kind: SH items, then small items (kGroupRows:
 // group of rows by group of rows), then RSR.  kX: the xyz items draw the rows' noise
 // from the values kept in X and subtract it, the opacity items count the rows
 // active after the step, and the tile's count is added to a.n_active.  kLarge:
-// the gradients of a sparse tile are read as ordinary lines (kLargeRows).
-template <int kTile, int kPrec, int kW, bool kX, bool kLarge>
+// the gradients of a sparse tile are read as ordinary lines (kLargeRows).  kOne:
+// an FP32 tile of up to two groups runs as one (kGroupRows).
+template <int kTile, int kPrec, int kW, bool kX, bool kLarge, bool kOne>
 __device__ __forceinline__ void tile_items(const StepArgs &a, const TileLists<kTile> &L, TileTerms<kTile> *X,
                                            const int nv, const int nr, const int rows)
 {
@@ -199,9 +200,9 @@ __device__ __forceinline__ void tile_items(const StepArgs &a, const TileLists<kT
     };
     if (kLarge && 4 * nv <= rows) {
         if constexpr (kLarge) run(std::true_type{}, 0, nv);
-    } else if constexpr (kPrec == GS_MOM_FP32) {
+    } else if (kPrec == GS_MOM_FP32 && (!kOne || nv > 2 * kGroupRows)) {
         for (int j0 = 0; j0 < nv; j0 += kGroupRows) run(std::false_type{}, j0, min(nv - j0, kGroupRows));
-    } else {
+    } else if constexpr (kPrec != GS_MOM_FP32 || kOne) {
         run(std::false_type{}, 0, nv);
     }
     const int e0 = kPrec == GS_MOM_FP32 ? 0 : kItems * nv, e_all = e0 + kItems * nr;
@@ -221,7 +222,7 @@ __device__ __forceinline__ void tile_items(const StepArgs &a, const TileLists<kT
 }
 
 // One tile: phase A, then its items.
-template <int kTile, int kPrec, int kW, bool kX = false, bool kLarge = false>
+template <int kTile, int kPrec, int kW, bool kX = false, bool kLarge = false, bool kOne = false>
 __device__ __forceinline__ void process_tile(const StepArgs &a, const int vis_src, const TileSpan span,
                                              TileLists<kTile> &L, TileTerms<kTile> *X = nullptr)
 {
@@ -230,7 +231,7 @@ __device__ __forceinline__ void process_tile(const StepArgs &a, const int vis_sr
     using S = State<kPrec>;
     int nv, nr;
     tile_decide<kTile, S::kRowBytes, S::kTByte, kX>(a, vis_src, span, L, X, nv, nr);
-    tile_items<kTile, kPrec, kW, kX, kLarge>(a, L, X, nv, nr, span.rows);
+    tile_items<kTile, kPrec, kW, kX, kLarge, kOne>(a, L, X, nv, nr, span.rows);
 }
 
 template <int kTile, int kMinBlocks, int kPrec, int kW, bool kLarge>
@@ -239,7 +240,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile(const StepArgs
     __shared__ TileLists<kTile> L;
     pdl_wait();
     prefetch_tile_ahead(a, vis_src);
-    process_tile<kTile, kPrec, kW, false, kLarge>(a, vis_src, tile_span(a, blockIdx.x), L);
+    process_tile<kTile, kPrec, kW, false, kLarge, !kLarge>(a, vis_src, tile_span(a, blockIdx.x), L);
     pdl_release();
 }
 
@@ -254,7 +255,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_terms(const St
     pdl_wait();
     prefetch_tile_ahead(a, vis_src);
     prefetch_tile_ahead_x(a);
-    process_tile<kTile, kPrec, kW, true, kLarge>(a, vis_src, tile_span(a, blockIdx.x), L, &X);
+    process_tile<kTile, kPrec, kW, true, kLarge, !kLarge>(a, vis_src, tile_span(a, blockIdx.x), L, &X);
     pdl_release();
 }
 
