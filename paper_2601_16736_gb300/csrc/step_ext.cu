@@ -408,6 +408,12 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_x(const StepAr
     using S = State<kPrec>;
     constexpr int kNsh = 48 / kW;
     __shared__ TileListsX<kTile> L;
+    // The next launch is let in at once for the 16-bit formats, at the end of the CTA
+    // (gs_internal.cuh) for FP32.  2 M rows, 10 % visible, end and start: noise on
+    // every row and AIU, FP16 block 194 and 185 us, BF16 151 and 148, hybrid 162 and
+    // 161, FP32 145 and 144; noise alone, FP16 128 and 129, BF16 106 and 108, hybrid
+    // 118 and 121, FP32 111 and 113.
+    if constexpr (kPrec != GS_MOM_FP32) pdl_release();
     pdl_wait();
     prefetch_tile_ahead(a, vis_src);
     prefetch_tile_ahead_x(a);
@@ -463,7 +469,7 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_x(const StepAr
         __syncthreads();
         if (threadIdx.x == 0 && L.active) atomicAdd(a.n_active, (unsigned long long)L.active);
     }
-    pdl_release();
+    if constexpr (kPrec == GS_MOM_FP32) pdl_release();
 }
 
 }  // namespace
