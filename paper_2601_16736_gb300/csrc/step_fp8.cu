@@ -687,48 +687,13 @@ __device__ __forceinline__ void f8_block_full(const StepArgs &a, const int vis_s
     }
 }
 
-// The blocks of a step on their full pass: tile = full0 + kF8FullEvery * i.
-// The others take their grow-only step.
-//
-// A scene of more than one wave takes two launches, first the full passes, then
-// the rest: with both in one kernel, the full pass's 40 KB of shared memory is
-// set aside for every block, at the expense of L1 (2 M rows, 20 % visible: 139 us
-// against 145).  The few full-pass CTAs let the next launch start as soon as
-// they run, so the two overlap; the blocks are distinct, so neither reads what
-// the other writes.
-template <int kT, int kMinBlocks>
-__global__ void __launch_bounds__(kT, kMinBlocks) step_fp8_full(const StepArgs a, const int vis_src, const int full0)
-{
-    __shared__ F8FullShared F;
-    pdl_release();
-    f8_block_full<kT>(a, vis_src, full0 + (int)kF8FullEvery * (int)blockIdx.x, F);
-}
-
-template <int kT>
-__device__ __forceinline__ void f8_grow_tile(const StepArgs &a, const int vis_src, const int tile, const int full0,
-                                             F8GrowShared &S)
-{
-    if ((uint32_t)tile % kF8FullEvery == (uint32_t)full0) return;
-    f8_prefetch_ahead(a, vis_src, tile);
-    const int nrow = (int)min((int64_t)kF8Tile, (int64_t)a.n_rows - (int64_t)tile * kF8Tile);
-    f8_block_grow<kT>(a, vis_src, tile, nrow, S);
-}
-
-// Launched with programmatic serialisation after step_fp8_full, which started
-// after all earlier work had completed; the last CTA waits for that launch to
-// complete, so that this one completes after it and whatever follows in the
-// stream sees both.
-template <int kT, int kMinBlocks>
-__global__ void __launch_bounds__(kT, kMinBlocks) step_fp8_grow(const StepArgs a, const int vis_src, const int full0)
-{
-    __shared__ F8GrowShared S;
-    f8_grow_tile<kT>(a, vis_src, (int)blockIdx.x, full0, S);
-    if (blockIdx.x == gridDim.x - 1) pdl_wait();
-}
-
-// A scene of at most one wave: one launch, the n_full longer CTAs first, in the
-// chain of programmatic launches (30 k rows, 88 % visible: 21.0 us against 23.3;
-// 30 %: 15.3 against 17.3).
+// One launch per step: the first n_full CTAs take the blocks on their full pass
+// (tile = full0 + kF8FullEvery * i), so that these longer CTAs start first; every
+// other CTA takes tile blockIdx.x - n_full on its grow-only step (returning at once
+// for the full-pass tiles).  A launch of its own for the full passes, whose 40 KB of
+// shared memory every CTA sets aside here, lost to this at every size above one wave:
+// 300 k rows, 10 % visible 20.3 us against 17.7, 750 k, 20 % 53.9 against 51.2, 2 M,
+// 20 % 127.4 against 124.9 (2 M, 30 %: 171.3 against 172.7).
 template <int kT, int kMinBlocks>
 __global__ void __launch_bounds__(kT, kMinBlocks) step_fp8(const StepArgs a, const int vis_src, const int full0,
                                                             const int n_full)
@@ -738,9 +703,14 @@ __global__ void __launch_bounds__(kT, kMinBlocks) step_fp8(const StepArgs a, con
         F8GrowShared grow;
     } sh;
     pdl_wait();
-    const int b = (int)blockIdx.x;
-    if (b < n_full) f8_block_full<kT>(a, vis_src, full0 + (int)kF8FullEvery * b, sh.full);
-    else f8_grow_tile<kT>(a, vis_src, b - n_full, full0, sh.grow);
+    const int b = (int)blockIdx.x, tile = b - n_full;
+    if (b < n_full) {
+        f8_block_full<kT>(a, vis_src, full0 + (int)kF8FullEvery * b, sh.full);
+    } else if ((uint32_t)tile % kF8FullEvery != (uint32_t)full0) {
+        f8_prefetch_ahead(a, vis_src, tile);
+        const int nrow = (int)min((int64_t)kF8Tile, (int64_t)a.n_rows - (int64_t)tile * kF8Tile);
+        f8_block_grow<kT>(a, vis_src, tile, nrow, sh.grow);
+    }
     pdl_release();
 }
 
@@ -998,29 +968,22 @@ __global__ void __launch_bounds__(kThreads, 3) reindex_fp8_kernel(
 // One CTA of 256 threads per block, 4 to an SM (64 registers), or of 512
 // threads, 2 to an SM, when those take every block at once: a small scene is
 // then as many threads wide as the chip holds, and each block is done in half
-// the passes (70 k rows: 29 us against 35; 2 M rows at 20 % visible, where the
-// work per block is too little for 512 threads: 190 against 135).
+// the passes (70 k rows: 0.83 of the time with 256 threads; 2 M rows at 20 %
+// visible, where the work per block is too little for 512: 1.4 times).
 cudaError_t launch_step_fp8(const StepArgs &a, int vis_src, cudaStream_t s)
 {
     if (a.n_rows <= 0) return cudaSuccess;
     static int s_res[64] = {};
-    const int resident = resident_ctas(reinterpret_cast<const void *>(step_fp8_grow<kThreads, kF8MinBlocks>), s_res);
+    const int resident = resident_ctas(reinterpret_cast<const void *>(step_fp8<kThreads, kF8MinBlocks>), s_res);
     const int n_tiles = (int)((a.n_rows + kF8Tile - 1) / kF8Tile);
     StepArgs b = a;
     b.tile_ahead = resident;
     // the tiles of this step's full pass: (iteration + tile) % kF8FullEvery == 0
     const int full0 = (int)((kF8FullEvery - (uint32_t)(a.k_ctr % kF8FullEvery)) % kF8FullEvery);
     const int n_full = full0 < n_tiles ? (n_tiles - full0 + (int)kF8FullEvery - 1) / (int)kF8FullEvery : 0;
-    if (n_tiles <= resident / 2)
-        return launch_pdl(step_fp8<2 * kThreads, kF8MinBlocks / 2>, (unsigned)(n_full + n_tiles), 2 * kThreads, s, b,
-                          vis_src, full0, n_full);
-    if (n_tiles <= resident || !n_full)
-        return launch_pdl(step_fp8<kThreads, kF8MinBlocks>, (unsigned)(n_full + n_tiles), kThreads, s, b, vis_src,
-                          full0, n_full);
-    step_fp8_full<kThreads, kF8MinBlocks><<<(unsigned)n_full, kThreads, 0, s>>>(b, vis_src, full0);
-    const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return launch_pdl(step_fp8_grow<kThreads, kF8MinBlocks>, (unsigned)n_tiles, kThreads, s, b, vis_src, full0);
+    const bool wide = n_tiles <= resident / 2;
+    auto k = wide ? step_fp8<2 * kThreads, kF8MinBlocks / 2> : step_fp8<kThreads, kF8MinBlocks>;
+    return launch_pdl(k, (unsigned)(n_full + n_tiles), (wide ? 2 : 1) * kThreads, s, b, vis_src, full0, n_full);
 }
 
 cudaError_t launch_export_fp8(const StateView &st, int32_t n, float *m_out, float *v_out, uint32_t *t_out,
