@@ -448,7 +448,6 @@ __device__ __forceinline__ void f8_block_grow(const StepArgs &a, const int vis_s
 struct F8FullShared {
     uint32_t cm[kF8Tile * kF8Row / 4], cv[kF8Tile * kF8Row / 4];
     __align__(16) float s_old[2][64], s_inv[2][64];
-    float s_new[2][64];
     uint32_t s_max[2][64];
     uint32_t s_wmax[kF8MaxThreads / 32][2][kF8Row / 4 - 1];
     uint8_t flg[kF8Tile];                     // bit 0 visible, bit 1 StSS-sampled
@@ -526,7 +525,6 @@ __device__ __forceinline__ void f8_block_full(const StepArgs &a, const int vis_s
     auto &cv = F.cv;
     auto &s_old = F.s_old;
     auto &s_inv = F.s_inv;
-    auto &s_new = F.s_new;
     auto &s_max = F.s_max;
     auto &s_wmax = F.s_wmax;
     auto &flg = F.flg;
@@ -643,7 +641,6 @@ __device__ __forceinline__ void f8_block_full(const StepArgs &a, const int vis_s
             if (e > eo) s = pow2f(so > 0.f ? min(e + kF8Headroom, 126) : e);
             else if (e <= eo - kF8Headroom - 1) s = pow2f(min(e + kF8Headroom, 126));
         }
-        s_new[w][c] = s;
         s_inv[w][c] = f8_inv(s);
         if (s != so) {
             (w ? a.vsc : a.msc)[tile * 64 + c] = s;
@@ -651,7 +648,6 @@ __device__ __forceinline__ void f8_block_full(const StepArgs &a, const int vis_s
         }
     } else if (tid < 2 * kF8Cols + 2) {
         const int w = tid - 2 * kF8Cols;     // the padding slot: encodes 0
-        s_new[w][kF8Cols] = 0.f;
         s_inv[w][kF8Cols] = 0.f;
     }
     __syncthreads();
