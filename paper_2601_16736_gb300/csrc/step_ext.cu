@@ -411,9 +411,11 @@ __global__ void __launch_bounds__(kThreads, kMinBlocks) step_tile_x(const StepAr
     // The next launch is let in at once for the 16-bit formats, at the end of the CTA
     // (gs_internal.cuh) for FP32.  2 M rows, 10 % visible, end and start: noise on
     // every row and AIU, FP16 block 194 and 185 us, BF16 151 and 148, hybrid 162 and
-    // 161, FP32 145 and 144; noise alone, FP16 128 and 129, BF16 106 and 108, hybrid
-    // 118 and 121, FP32 111 and 113.
-    if constexpr (kPrec != GS_MOM_FP32) pdl_release();
+    // 161; noise alone, FP16 128 and 129, BF16 106 and 108, hybrid 118 and 121, FP32
+    // 111 and 113.  FP32 with both terms gains by the end up to 1 M rows (600 k, 10 %:
+    // 50.2 and 51.4) and loses in large scenes (6 M: 425 and 418), so there it is at
+    // the start as well.
+    if (kPrec != GS_MOM_FP32 || (kLarge && a.aiu && a.noise)) pdl_release();
     pdl_wait();
     prefetch_tile_ahead(a, vis_src);
     prefetch_tile_ahead_x(a);
