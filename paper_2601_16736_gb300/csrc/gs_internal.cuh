@@ -22,10 +22,10 @@ namespace gs {
 // the lines it touches: with m and v in arrays of their own a hybrid row
 // (2 x 160 B) touched four lines and an FP8 row (2 x 64 B) two; side by side
 // they touch three and one.  The v row's address is the m row's plus a
-// constant, which the items fold into their loads and stores.  Per step, side
-// by side against separate arrays: hybrid 239 us against 257 (6 M rows, 10 %
-// visible), FP16 block 178 against 183 (3 M, 20 %), FP8 154 against 160 (2 M,
-// 20 %), FP32 and BF16 level.
+// constant, which the items fold into their loads and stores.  When it was
+// changed, a step with them side by side took 0.93 of its time with separate
+// arrays for hybrid (6 M rows, 10 % visible), 0.97 for FP16 block (3 M, 20 %),
+// 0.96 for FP8 (2 M, 20 %), and the same for FP32 and BF16.
 // Slot order inside an m or v row:
 //   0-47  SH (same column order as the sh group)
 //   48-51 rotation, 52-54 xyz, 55-57 scale, 58 opacity
@@ -273,13 +273,17 @@ struct BatchParams {
 // Programmatic dependent launch.  The kernels of this library are launched
 // with programmatic stream serialisation: a kernel may be scheduled before the
 // kernel ahead of it in the stream has completed, and waits (pdl_wait) until that
-// one has and its writes are visible, before touching any data.  A CTA lets the
-// next launch in (pdl_release) when its own work is done, so the next kernel's
-// CTAs take their places as the last ones of this grid finish and are resident
-// when it ends.  Letting them in at the start instead places them wherever the
-// grid leaves room, beside CTAs at work, so they are spread unevenly in their
-// turn (1 M rows, 30 % visible: 109.1 us a step against 107.6; 20 k rows: 9.9
-// against 7.8), and made a checkpoint's export after its import 4 % slower.
+// one has and its writes are visible, before touching any data.  Every thread of
+// every CTA waits, so that a kernel completes after all that were ahead of it.
+// A CTA lets the next launch in (pdl_release) when its own work is done, so the
+// next kernel's CTAs take their places as the last ones of this grid finish and are
+// resident when it ends.  Letting them in at the start instead places them wherever
+// the grid leaves room, beside CTAs at work, so they are spread unevenly in their
+// turn (when it was changed, 1 M rows, 30 % visible: 109.1 us a step against 107.6;
+// 20 k rows: 9.9 against 7.8), and made a checkpoint's export after its import 4 %
+// slower.  Two kinds of kernel release at the start all the same: the one thread
+// that clears the visibility count, whose successor should be resident by then, and
+// the extended step where that is faster (step_tile_x).
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

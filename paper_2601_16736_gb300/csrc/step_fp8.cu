@@ -1,11 +1,12 @@
 // FP8 (e4m3) moments with per-256-row block scales.
 //
-// Storage: m and v rows of 64 bytes side by side (one 128-B line a primitive), the 59 e4m3 codes in work-chunk order
-// (SH 0-47, rotation 48-51, xyz 52-54, opacity 55, scale 56-58; byte 59 is
-// padding and bytes 60-63 of the m row hold the step counter t), so that
-// each 4-value work chunk is one 32-bit word; and for every block of 256
-// rows one FP32 scale per slot for m and one for v (a power of two, 0 for a
-// slot that is zero throughout the block).  A value is code x scale.
+// Storage: m and v rows of 64 bytes side by side (one 128-B line a primitive),
+// the 59 e4m3 codes in work-chunk order (SH 0-47, rotation 48-51, xyz 52-54,
+// opacity 55, scale 56-58; byte 59 is padding and bytes 60-63 of the m row hold
+// the step counter t), so that each 4-value work chunk is one 32-bit word; and
+// for every block of 256 rows one FP32 scale per slot for m and one for v (a
+// power of two, 0 for a slot that is zero throughout the block).  A value is
+// code x scale.
 //
 // A block's scale is a power of two that keeps the largest magnitude of its
 // slot within e4m3's finite range (448).  Sparse Adam updates only the
@@ -840,7 +841,8 @@ __global__ void __launch_bounds__(kThreads, 2) import_fp8_kernel(uint4 *__restri
 // maxima and the one that re-encodes, so each state row is read once.  2 M rows:
 // 226 us against 351 with a thread per value and an atomic maximum for each
 // (floor 70: the conversions now take the time; 512 threads of 4 rows, reading
-// the scales for each: 314; two CTAs an SM without spills: 256).
+// the scales for each: 314).  Three CTAs an SM spill a few of a thread's registers
+// (80 B stored, 136 B loaded); two, which do not, took 256.
 __device__ __forceinline__ void f8_scales16(const float *sc, int32_t blk, float *s)
 {
 #pragma unroll
